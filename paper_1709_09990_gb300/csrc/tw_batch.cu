@@ -30,8 +30,7 @@ __global__ void __launch_bounds__(kBatchWarps * 32, 6)
                         unsigned long long* out_keys, uint32_t* out_parent, BatchCounters* ctr, int max_probes) {
   using K = unsigned long long;
   __shared__ K sAdj[kBatchWarps][64];
-  __shared__ K sState[kBatchWarps][32];
-  __shared__ uint16_t sQueue[kBatchWarps][32 * 64];
+  __shared__ core::WarpScratch<K> sScratch[kBatchWarps];
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
   const unsigned long long stride = (unsigned long long)gridDim.x * kBatchWarps;
@@ -39,8 +38,18 @@ __global__ void __launch_bounds__(kBatchWarps * 32, 6)
   BatchSeg sg{};
   K valid = 0;
   core::LevelOut<K, true> out{};
+  core::WarpScratch<K>& w = sScratch[warp];
+  int staged = 0;
+  unsigned long long generated = 0;
+  // the warp's staged sets and pair count go to its graph's list and counter
+  auto finish_graph = [&]() {
+    core::flush_stage<K, true, false>(w, staged, lane, out, nullptr, 0ull);
+    core::add_warp_count(generated, lane, &ctr[cur].generated);
+    generated = 0;
+  };
   for (unsigned long long c = (unsigned long long)blockIdx.x * kBatchWarps + warp; c < total_chunks; c += stride) {
     if (cur < 0 || c < chunk_begin[cur] || c >= chunk_begin[cur + 1]) {
+      if (cur >= 0) finish_graph();
       int lo = 0, hi = nseg - 1;  // last s with chunk_begin[s] <= c
       while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
@@ -68,14 +77,16 @@ __global__ void __launch_bounds__(kBatchWarps * 32, 6)
     const unsigned long long idx = local * 32ull + lane;
     const bool active = idx < sg.in_count;
     const K S = active ? keys[sg.in_off + idx] : valid;
-    const K feas = active ? core::feasible_extensions<K>(S, sAdj[warp], valid, valid, sg.k) : 0ull;
-    const int total = core::build_queue<K>(S, feas, lane, sState[warp], sQueue[warp]);
-    if (lane == 0 && total) atomicAdd(&ctr[cur].generated, (unsigned long long)total);
+    core::Candidates<K> cand = core::start_chunk<K, true>(S, active, sAdj[warp], valid, valid, sg.n, sg.k, lane, w);
     out.parent_base = (uint32_t)(local * 32ull);
-    core::insert_queue<K, true>(sQueue[warp], sState[warp], total, lane, table + sg.t_off, sg.t_slots, max_probes,
-                                out);
-    __syncwarp();
+    do {
+      const int total = core::build_queue<K>(cand, lane, w);
+      generated += (unsigned long long)core::search_insert<K, true>(w, total, staged, lane, sAdj[warp], sg.k,
+                                                                    table + sg.t_off, sg.t_slots, max_probes, out);
+      __syncwarp();
+    } while (__any_sync(kFull, core::any_left(cand)));
   }
+  if (cur >= 0) finish_graph();
 }
 
 // Copies segment s of (keys, parents) from src to dst; src_off == ~0 writes

@@ -375,7 +375,9 @@ int run_batch(tw_ctx* c, const std::vector<HostGraph>& graphs, const std::vector
         --running;
         continue;
       }
-      const unsigned long long slots = std::max<unsigned long long>(64, (unsigned long long)std::ceil(table_est * 2.0));
+      // (whole 32-byte sectors: every graph's table starts at one)
+      const unsigned long long slots =
+          (std::max<unsigned long long>(64, (unsigned long long)std::ceil(table_est * 2.0)) + 3ull) & ~3ull;
       // (more than 90% of the slots filled re-runs the level with a larger
       // table, so the output never needs more room than that)
       unsigned long long oc =

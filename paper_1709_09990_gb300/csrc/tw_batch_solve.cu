@@ -77,8 +77,8 @@ __device__ void block_fingerprint(const K* keys, unsigned long long count, unsig
 // the levels outgrow the workspace; else *yes and *last (the final level).
 // With fp_sum / fp_xor (decide mode) the level fingerprints are written.
 template <int kWarps>
-__device__ __noinline__ bool block_decide(const BatchSolveArgs& a, const K* adj, int n, int k, Work& w, K* sAdj, K* sState,
-                             uint16_t* sQueue, unsigned long long* sRed, bool* yes, int* last,
+__device__ __noinline__ bool block_decide(const BatchSolveArgs& a, const K* adj, int n, int k, Work& w, K* sAdj,
+                             core::WarpScratch<K>* sScratch, unsigned long long* sRed, bool* yes, int* last,
                              unsigned long long* stats, unsigned long long* fp_sum, unsigned long long* fp_xor) {
   for (int t = 0; t < 2; ++t) {
     for (unsigned long long j = threadIdx.x; j < w.dirty[t]; j += blockDim.x) w.table[t][j] = kones<K>();
@@ -131,7 +131,7 @@ __device__ __noinline__ bool block_decide(const BatchSolveArgs& a, const K* adj,
       p.mmw = 0;
       p.ranges = 1;
       p.range = 0;
-      core::expand_level<K, kWarps, TW_INSERT_UNROLL, false, false, true, true>(p, sAdj, sState, sQueue);
+      core::expand_level<K, kWarps, false, false, true, true>(p, sAdj, sScratch);
       for (unsigned long long j = threadIdx.x; j < w.dirty[1 - t]; j += blockDim.x) w.table[1 - t][j] = kones<K>();
       w.dirty[1 - t] = 0;
       w.dirty[t] = max(w.dirty[t], slots);
@@ -174,8 +174,7 @@ __device__ __noinline__ bool block_decide(const BatchSolveArgs& a, const K* adj,
 template <int kWarps>
 __global__ void __launch_bounds__(kWarps * 32, 24 / kWarps) batch_solve_kernel(const BatchSolveArgs a) {
   __shared__ K sAdj[64];
-  __shared__ K sState[kWarps * 32];
-  __shared__ uint16_t sQueue[kWarps * 32 * 64];
+  __shared__ core::WarpScratch<K> sScratch[kWarps];
   __shared__ unsigned long long sRed[2 * kWarps];
   __shared__ K sWalk;
   __shared__ int sFound;
@@ -205,7 +204,7 @@ __global__ void __launch_bounds__(kWarps * 32, 24 / kWarps) batch_solve_kernel(c
     if (a.decide_mode) {
       unsigned long long* fs = a.fp_sum ? a.fp_sum + (size_t)g * 129 : nullptr;
       unsigned long long* fx = a.fp_xor ? a.fp_xor + (size_t)g * 129 : nullptr;
-      const bool ok = block_decide<kWarps>(a, adj, n, a.k_start[g], w, sAdj, sState, sQueue, sRed, &yes, &last,
+      const bool ok = block_decide<kWarps>(a, adj, n, a.k_start[g], w, sAdj, sScratch, sRed, &yes, &last,
                                            stats, fs, fx);
       ++runs;
       if (threadIdx.x == 0) {
@@ -224,7 +223,7 @@ __global__ void __launch_bounds__(kWarps * 32, 24 / kWarps) batch_solve_kernel(c
     int yes_min = INT_MAX, no_max = lb - 1, yes_in_arena = -1;
     bool ok = true;
     for (;;) {
-      ok = block_decide<kWarps>(a, adj, n, k, w, sAdj, sState, sQueue, sRed, &yes, &last, stats, nullptr, nullptr);
+      ok = block_decide<kWarps>(a, adj, n, k, w, sAdj, sScratch, sRed, &yes, &last, stats, nullptr, nullptr);
       ++runs;
       if (!ok) break;
       if (yes) {
@@ -239,7 +238,7 @@ __global__ void __launch_bounds__(kWarps * 32, 24 / kWarps) batch_solve_kernel(c
     }
     if (ok && yes_in_arena != yes_min) {
       // the last run was a no: run the yes at tw again for its levels
-      ok = block_decide<kWarps>(a, adj, n, yes_min, w, sAdj, sState, sQueue, sRed, &yes, &last, stats, nullptr,
+      ok = block_decide<kWarps>(a, adj, n, yes_min, w, sAdj, sScratch, sRed, &yes, &last, stats, nullptr,
                                 nullptr);
       ++runs;
     }

@@ -7,27 +7,23 @@
 // table and appended to L_{i+1} together with the predecessor vertex v.
 //
 // GB300 mapping.  A warp takes 32 consecutive states (coalesced key loads).
-//  1. Thread-per-state: the components of G[S] are found by a bitset flood
-//     fill over the adjacency rows held in shared memory, one row read per
-//     vertex of S at most.  Each component C contributes its outer boundary
-//     B_C = N(C) \ S.
-//     Then Q(S, v) = (N(v) u U{B_C : v in B_C}) \ (S u {v}), the bitset form
-//     of the depth-first search inside Listing 1: a vertex outside S
-//     is reached from v through S exactly when it borders a component of G[S]
-//     that v borders.  Components with |B_C| >= k+2 make every v in B_C
-//     infeasible at once; up to 8 other boundaries stay in registers, and a
-//     state with more falls back to a flood fill per candidate v.  Only the
-//     canonical candidates are tested: v below min(S), or v on the boundary
-//     of the component of min(S); that generates every set of L_{i+1} (see
-//     feasible_extensions) from about a third as many parents.  The flood
-//     fill is lazy: the component of min(S) first, then only the components
-//     next to a candidate that passes |N(v) \ S| <= k.
-//  2. Warp-cooperative insert: the feasible (S, v) pairs of the 32 states are
-//     packed into a per-warp shared-memory queue, and the whole warp inserts
-//     32 of them at a time with one 4/8/16-byte compare-and-swap each, so
-//     lanes do not idle on states with few extensions.
-//  3. The winners of a round append (S u {v}, v) to L_{i+1} with one atomic
-//     add per warp.
+//  1. Thread per state: the component of G[S] that holds min(S) is found by a
+//     bitset flood fill over the adjacency rows in shared memory, and the
+//     canonical candidates (v below min(S), or v on that component's boundary;
+//     that generates every set of L_{i+1}, see cheap_candidates) that pass a
+//     cheap lower bound of |Q(S, v)| go to the warp's queue.
+//  2. Pair per lane: each queued (S, v) is searched on its own (the bitset form
+//     of the search inside Listing 1, started from the component of min(S) when
+//     v borders it) and, if feasible, probed in the exact hash table, a 32-byte
+//     sector per load.  Pairs that need no search come first in the queue.
+//  3. New sets wait in shared memory and are appended to L_{i+1} with one atomic
+//     add per 200 or so: all adds of a level go to one counter.
+// The kernel is bound by instruction issue (62% of the issue slots at the peak
+// level of the geometric n=40 graph) and L2 round trips; the expand time of that
+// graph's 79.4 M sets is 7.7 ms, against 11.1 ms with a search per state (all
+// components of G[S] first, then the candidates) and slot-by-slot
+// compare-and-swaps, of which 3.4 ms went to lanes waiting for the warp's
+// longest probe sequence and to the counter.
 #include <cuda_runtime.h>
 
 #include "tw_expand_core.cuh"
@@ -41,69 +37,63 @@ using core::ExpandParams;
 using core::ResidentWarps;
 using core::kFull;
 
-template <class K, int kWarps, int U, bool kMMW = false, bool kRanged = false>
+template <class K, int kWarps, bool kMMW = false>
 __global__ void __launch_bounds__(kWarps * 32, ResidentWarps<K>::value / kWarps)
     expand_insert_kernel(const ExpandParams<K> p) {
-  constexpr int kBits = KeyTraits<K>::kBits;
-  __shared__ K sAdj[kBits];
-  __shared__ K sState[kWarps * 32];
-  __shared__ uint16_t sQueue[kWarps * 32 * kBits];
-  core::expand_level<K, kWarps, U, kMMW, kRanged>(p, sAdj, sState, sQueue);
+  __shared__ K sAdj[KeyTraits<K>::kBits];
+  __shared__ core::WarpScratch<K> sScratch[kWarps];
+  core::expand_level<K, kWarps, kMMW>(p, sAdj, sScratch);
 }
 
 // One hash range of a level whose table is built slice by slice; the output
 // list may continue in a second buffer (out_tail from position out_split on).
-template <class K, int U>
+template <class K>
 __global__ void __launch_bounds__(4 * 32, ResidentWarps<K>::value / 4)
     expand_ranged_kernel(const ExpandParams<K> p, K* out_tail, unsigned long long out_split) {
-  constexpr int kBits = KeyTraits<K>::kBits;
-  __shared__ K sAdj[kBits];
-  __shared__ K sState[4 * 32];
-  __shared__ uint16_t sQueue[4 * 32 * kBits];
-  core::expand_level<K, 4, U, false, true>(p, sAdj, sState, sQueue, 0u, 0u, out_tail, out_split);
+  __shared__ K sAdj[KeyTraits<K>::kBits];
+  __shared__ core::WarpScratch<K> sScratch[4];
+  core::expand_level<K, 4, false, true>(p, sAdj, sScratch, 0u, 0u, out_tail, out_split);
 }
 
 // A ranged launch: 4 warps per block, one block per SM slot.
-template <class K, int U>
+template <class K>
 cudaError_t launch_ranged(const ExpandParams<K>& p, K* out_tail, unsigned long long out_split,
                           unsigned long long blocks_needed, cudaStream_t s) {
   int per_sm = 0, dev = 0, sms = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, expand_ranged_kernel<K, U>, 128, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, expand_ranged_kernel<K>, 128, 0);
   unsigned long long grid = (unsigned long long)sms * (per_sm > 0 ? per_sm : 1);
   if (grid > blocks_needed) grid = blocks_needed;
-  expand_ranged_kernel<K, U><<<(int)grid, 128, 0, s>>>(p, out_tail, out_split);
+  expand_ranged_kernel<K><<<(int)grid, 128, 0, s>>>(p, out_tail, out_split);
   return cudaGetLastError();
 }
 
-template <class K, int kWarps, int U>
-cudaError_t launch_expand_u(const ExpandParams<K>& p, unsigned long long blocks_needed, int grid, KeyClass kc,
+template <class K, int kWarps>
+cudaError_t launch_direct(const ExpandParams<K>& p, unsigned long long blocks_needed, int grid, KeyClass kc,
                             cudaStream_t s) {
   if (grid <= 0) {
-    // resident blocks per SM x SMs, cached per (device, width, warps, U)
-    static thread_local int cached_dev = -1, cached_grid[3][3][2] = {{{0}}};
+    // resident blocks per SM x SMs, cached per (device, width, warps)
+    static thread_local int cached_dev = -1, cached_grid[3][3] = {{0}};
     int dev = 0;
     cudaGetDevice(&dev);
     const int wi = kWarps == 2 ? 0 : (kWarps == 4 ? 1 : 2);
-    const int ui = U == TW_INSERT_UNROLL ? 0 : 1;
     if (cached_dev != dev) {
-      for (auto& a : cached_grid)
-        for (auto& r : a)
-          for (int& x : r) x = 0;
+      for (auto& r : cached_grid)
+        for (int& x : r) x = 0;
       cached_dev = dev;
     }
-    int& g = cached_grid[(int)kc][wi][ui];
+    int& g = cached_grid[(int)kc][wi];
     if (g == 0) {
       int sms = 0, per_sm = 0;
       cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, expand_insert_kernel<K, kWarps, U>, kWarps * 32, 0);
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, expand_insert_kernel<K, kWarps>, kWarps * 32, 0);
       g = sms * (per_sm > 0 ? per_sm : 1);
     }
     grid = g;
   }
   if ((unsigned long long)grid > blocks_needed) grid = (int)blocks_needed;
-  expand_insert_kernel<K, kWarps, U><<<grid, kWarps * 32, 0, s>>>(p);
+  expand_insert_kernel<K, kWarps><<<grid, kWarps * 32, 0, s>>>(p);
   return cudaGetLastError();
 }
 
@@ -131,28 +121,21 @@ cudaError_t launch_expand_t(const ExpandLaunch& a, cudaStream_t s) {
   const unsigned long long blocks_needed = (chunks + kWarps - 1) / kWarps;
   if (a.ranges > 0) {
     const unsigned long long need4 = (chunks + 3) / 4;
-    K* tail = static_cast<K*>(a.out_tail);
-    if (a.table_slots * sizeof(K) > core::kDeepTableBytes)
-      return launch_ranged<K, 2 * TW_INSERT_UNROLL>(p, tail, a.out_split, need4, s);
-    return launch_ranged<K, TW_INSERT_UNROLL>(p, tail, a.out_split, need4, s);
+    return launch_ranged<K>(p, static_cast<K*>(a.out_tail), a.out_split, need4, s);
   }
   if (a.mmw) {
     // minor-min-width pruning (opt-in): its own instantiation, 4 warps
     int per_sm = 0, dev = 0, sms = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, expand_insert_kernel<K, 4, TW_INSERT_UNROLL, true>, 128, 0);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, expand_insert_kernel<K, 4, true>, 128, 0);
     unsigned long long grid = (unsigned long long)sms * (per_sm > 0 ? per_sm : 1);
     const unsigned long long need = (chunks + 3) / 4;
     if (grid > need) grid = need;
-    expand_insert_kernel<K, 4, TW_INSERT_UNROLL, true><<<(int)grid, 128, 0, s>>>(p);
+    expand_insert_kernel<K, 4, true><<<(int)grid, 128, 0, s>>>(p);
     return cudaGetLastError();
   }
-  // Tables far larger than L2 miss on most probes: keep twice as many
-  // compare-and-swaps in flight per lane there.
-  if (a.table_slots * sizeof(K) > core::kDeepTableBytes)
-    return launch_expand_u<K, kWarps, 2 * TW_INSERT_UNROLL>(p, blocks_needed, a.grid, a.kc, s);
-  return launch_expand_u<K, kWarps, TW_INSERT_UNROLL>(p, blocks_needed, a.grid, a.kc, s);
+  return launch_direct<K, kWarps>(p, blocks_needed, a.grid, a.kc, s);
 }
 
 template <class K>

@@ -15,20 +15,13 @@ namespace tw {
 namespace core {
 
 constexpr unsigned kFull = 0xffffffffu;
-constexpr int kMaxComps = 8;
-#ifndef TW_INSERT_UNROLL
-#define TW_INSERT_UNROLL 4  // compare-and-swaps in flight per lane (L2-resident tables)
-#endif
-// Tables larger than this many bytes (about twice the L2) miss in L2 on most
-// probes; their levels run with twice as many compare-and-swaps in flight.
-constexpr unsigned long long kDeepTableBytes = 256ull << 20;
-
-// Resident warps per SM the register allocation must allow: 32 for the 32-
-// and 64-bit kernels (at most 64 registers per thread, measured fastest on
-// GB300), 16 for the 128-bit kernel.
+// Resident warps per SM the register allocation must allow: 40 for the 32-bit
+// kernel (on a geometric n=25 graph 1.67 ms of expand time against 1.77 with
+// 32), 32 for the 64-bit one (with 40 it is 0.5% to 2% slower), 16 for the
+// 128-bit one.
 template <class K>
 struct ResidentWarps {
-  static constexpr int value = KeyTraits<K>::kBits <= 64 ? 32 : 16;
+  static constexpr int value = KeyTraits<K>::kBits <= 32 ? 40 : KeyTraits<K>::kBits <= 64 ? 32 : 16;
 };
 
 // Home slot of a hash: the high word of hash * slots (uniform over [0, slots)
@@ -37,171 +30,100 @@ __device__ __forceinline__ unsigned long long home_slot(unsigned long long h, un
   return __umul64hi(h, slots);
 }
 
-// Floods the component of G[S] that contains the vertices of todo (taken out
-// of rem, the vertices of S not yet in a component) over the adjacency rows in
-// shared memory; returns its outer boundary N(C) \ S and adds the component's
-// vertices to *comp.
+// The component of G[S] that holds min(S) and its outer boundary N(comp) \ S
+// (both empty for S = {}), by a bitset flood fill over the adjacency rows in
+// shared memory.
 template <class K>
-__device__ __forceinline__ K flood_component(K todo, K& rem, const K S, const K* __restrict__ sAdj, K* comp) {
-  K bnd = kzero<K>();
-  while (!kempty(todo)) {
-    const K b = klsb(todo);
-    todo ^= b;
+__device__ __forceinline__ void min_component(const K S, const K* __restrict__ sAdj, K& comp, K& bnd) {
+  comp = kzero<K>();
+  K q = kzero<K>();
+  K front = klsb(S);
+  while (!kempty(front)) {
+    const K b = klsb(front);
     const K r = sAdj[kindex(b)];
-    bnd |= r;
-    const K nw = r & rem;  // unvisited vertices of S next to the component
-    rem ^= nw;
-    todo |= nw;
-    if (comp) *comp |= nw;
+    q |= r;
+    comp |= b;
+    front = (front | r) & S & ~comp;
   }
-  return bnd & ~S;
+  bnd = q & ~S;
 }
 
-// Adds the boundary of one more component of G[S] to the registers of
-// feasible_extensions: a boundary with |B_C| >= k+2 rules out all of B_C;
-// up to kMaxComps others are kept; beyond that the caller falls back to a
-// flood fill per candidate.
-template <class K>
-__device__ __forceinline__ void keep_boundary(const K bnd, const int k, K (&comp_b)[kMaxComps], int& nc, bool& many,
-                                              K& dead, K& bordered) {
-  const int bs = kpopc(bnd);
-  if (bs >= k + 2) {
-    dead |= bnd;
-  } else if (bs > 0) {
-    if (nc < kMaxComps) {
-#pragma unroll
-      for (int c = 0; c < kMaxComps; ++c)
-        if (c == nc) comp_b[c] = bnd;
-      ++nc;
-      bordered |= bnd;
-    } else {
-      many = true;
-    }
-  }
-}
-
-// |Q(S, v)| <= k for one candidate v (bit vb, row nv = N(v)), given the
-// boundaries of the components of G[S] that v may border.
-template <class K>
-__device__ __forceinline__ bool q_within(const K S, const K vb, const K nv, K q, const K* __restrict__ sAdj,
-                                         const int k, const K (&comp_b)[kMaxComps], const int nc, const bool many,
-                                         const K bordered) {
-  if (!many) {
-    if (!kempty(bordered & vb)) {
-#pragma unroll
-      for (int c = 0; c < kMaxComps; ++c) {
-        if (c >= nc) break;
-        if (!kempty(comp_b[c] & vb)) q |= comp_b[c];
-      }
-    }
-  } else {
-    K vis = nv & S;
-    K front = vis;
-    while (!kempty(front)) {
-      const K b = klsb(front);
-      front ^= b;
-      const K r = sAdj[kindex(b)];
-      q |= r & ~S;
-      const K nw = r & S & ~vis;
-      vis |= nw;
-      front |= nw;
-    }
-  }
-  q &= ~vb;
-  return kpopc(q) <= k;
-}
-
-// The set of vertices v outside S with |Q(S, v)| <= k (thread per state).
+// The candidates v of state S (thread per state) that pass the cheap test: a
+// lower bound of |Q(S, v)| from v's own row and, when v borders the component
+// comp0 of min(S), that component's boundary b0, is at most k.
 //
-// The components of G[S] are found by a bitset flood fill over the adjacency
-// rows in shared memory; each component C gives its outer boundary
-// B_C = N(C) \ S.  A vertex outside S is reachable from v through S exactly
-// when it borders a component that v borders, so
-// Q(S, v) = (N(v) u U{B_C : v in B_C}) \ (S u {v}) - the bitset form of the
-// search of Listing 1.  A boundary with |B_C| >= k+2 rules out all of B_C at
-// once; up to kMaxComps other boundaries stay in registers, and a state with
-// more falls back to a flood fill per candidate.
-//
-// With kCanonical only the canonical extensions are returned: the v that lie
+// With kCanonical only the canonical extensions are candidates: the v that lie
 // in the component of G[S u {v}] holding the lowest vertex of S u {v}, i.e.
-// v below min(S) or v in the boundary of the component of min(S).  The level
-// sets stay exactly those of Listing 1: Q(S, v) depends only on v's component
-// of G[S u {v}] (a path from v whose interior lies in S never leaves it), so
-// a set is feasible iff each of its components is, and a feasible set T is
-// reached from T \ {u} with u the last vertex of a feasible ordering of T's
-// lowest-vertex component.  Each new set is then produced by far fewer
-// parents, which cuts the candidate tests and the table probes (on the
-// geometric n=40 benchmark graph 3.3x fewer pairs).  The canonical search is
-// also lazy: it floods the component of min(S) first, which fixes the
-// candidates, and then only the components that border a candidate passing
-// the |N(v) \ S| <= k test.
-template <class K, bool kCanonical = true>
-__device__ __forceinline__ K feasible_extensions(const K S, const K* __restrict__ sAdj, const K valid,
-                                                 const K allowed, const int k) {
-  K comp_b[kMaxComps];
-#pragma unroll
-  for (int c = 0; c < kMaxComps; ++c) comp_b[c] = kzero<K>();
-  int nc = 0;
-  bool many = false;
-  K dead = kzero<K>();
-  K bordered = kzero<K>();  // union of the kept boundaries
-  K rem = S;                // vertices of S not yet in a component
-  K cand;
-  if (kCanonical) {
-    K b0 = kzero<K>();  // boundary of the component of min(S)
-    if (!kempty(S)) {
-      const K first = klsb(S);
-      rem ^= first;
-      b0 = flood_component<K>(first, rem, S, sAdj, nullptr);
-    }
-    cand = valid & allowed & ~S & (kbelow_lowest(S) | b0);
-    if (kpopc(b0) >= k + 2) {
-      cand &= ~b0;
-    } else if (!kempty(b0)) {
-      comp_b[0] = b0;
-      nc = 1;
-      bordered = b0;
-    }
-    // keep the candidates that pass the cheap test; flood only the
-    // components of S next to them
-    K pre = kzero<K>(), need = kzero<K>();
-    for (K c = cand; !kempty(c);) {
-      const K vb = klsb(c);
-      c ^= vb;
-      const K nv = sAdj[kindex(vb)];
-      if (kpopc(nv & ~S) > k) continue;
-      pre |= vb;
-      need |= nv;
-    }
-    need &= rem;
-    while (!kempty(need)) {
-      const K start = klsb(need);
-      rem ^= start;
-      K comp = start;
-      const K bnd = flood_component<K>(start, rem, S, sAdj, &comp);
-      need &= ~comp;
-      keep_boundary<K>(bnd, k, comp_b, nc, many, dead, bordered);
-    }
-    cand = pre & ~dead;
-  } else {
-    while (!kempty(rem)) {
-      const K start = klsb(rem);
-      rem ^= start;
-      const K bnd = flood_component<K>(start, rem, S, sAdj, nullptr);
-      keep_boundary<K>(bnd, k, comp_b, nc, many, dead, bordered);
-    }
-    cand = valid & allowed & ~S & ~dead;
-  }
-  K feas = kzero<K>();
+// v below min(S) or v in b0.  The level sets stay exactly those of Listing 1:
+// Q(S, v) depends only on v's component of G[S u {v}] (a path from v whose
+// interior lies in S never leaves it), so a set is feasible iff each of its
+// components is, and a feasible set T is reached from T \ {u} with u the last
+// vertex of a feasible ordering of T's lowest-vertex component.  Each new set
+// is then produced by far fewer parents (on the geometric n=40 benchmark graph
+// 3.3x fewer pairs).
+//
+// Candidates that border no other component of G[S] (two of three on the
+// geometric n=40 graph) are settled by the test (done); the others still need
+// the search (search).
+template <class K>
+struct Candidates {
+  K done, search;
+};
+template <class K, bool kCanonical>
+__device__ __forceinline__ Candidates<K> cheap_candidates(const K S, const K comp0, const K b0,
+                                                          const K* __restrict__ sAdj, const K valid, const K allowed,
+                                                          const int k) {
+  K cand = valid & allowed & ~S;
+  if (kCanonical) cand &= kbelow_lowest(S) | b0;
+  Candidates<K> c{kzero<K>(), kzero<K>()};
   while (!kempty(cand)) {
     const K vb = klsb(cand);
     cand ^= vb;
     const K nv = sAdj[kindex(vb)];
-    const K q = nv & ~S;
-    if (kpopc(q) > k) continue;
-    if (q_within<K>(S, vb, nv, q, sAdj, k, comp_b, nc, many, bordered)) feas |= vb;
+    K t = nv, visit = nv & S;
+    int most = k;
+    if (kCanonical && !kempty(b0 & vb)) {
+      t |= b0;
+      visit &= ~comp0;
+      most = k + 1;  // (b0 holds v itself)
+    }
+    if (kpopc(t & ~S) <= most) {
+      if (kempty(visit))
+        c.done |= vb;
+      else
+        c.search |= vb;
+    }
   }
-  return feas;
+  return c;
+}
+
+// Is |Q(S, v)| <= k?  The search of Listing 1 as a bitset flood fill: it starts
+// from N(v) and, when v borders the component of min(S) (v in b0), from that
+// whole component at once (comp0, boundary b0), visits the vertices of S
+// reachable from v and gathers their rows; it stops as soon as the vertices
+// gathered outside S u {v} exceed k.
+template <class K>
+__device__ __forceinline__ bool extension_feasible(const K S, const K comp0, const K b0, const int v,
+                                                   const K* __restrict__ sAdj, const int k) {
+  const K vb = kbit<K>(v);
+  const K out = ~(S | vb);
+  K q = sAdj[v];
+  K done = ~S;  // vertices that need no visit: those outside S and those visited
+  if (!kempty(b0 & vb)) {
+    done |= comp0;
+    q |= b0;
+  }
+  K front = q & ~done;
+  bool within;
+  // (one way out of the loop, so that the warp's lanes meet again after it)
+  while ((within = kpopc(q & out) <= k) && !kempty(front)) {
+    const K b = klsb(front);
+    const K r = sAdj[kindex(b)];
+    q |= r;
+    done |= b;
+    front = (front | r) & ~done;
+  }
+  return within;
 }
 
 // Warp-wide minimum of (d, v), lowest v on ties; v < 0 means none.
@@ -312,43 +234,47 @@ __device__ __forceinline__ bool mmw_exceeds(const K S, const K* __restrict__ sAd
   return false;
 }
 
-// Drops the extensions of every state of the warp whose remaining graph has
-// a minor-min-width bound above k (the warp examines its states one by one).
+// Has this lane's state, if it is one of the extendable ones, a remaining graph
+// with a minor-min-width bound above k?  (The warp examines its states one by
+// one.)
 template <class K>
-__device__ __forceinline__ K mmw_filter(const K S, K feas, const K* __restrict__ sAdj, const int n, const int k,
-                                        const int lane) {
-  unsigned pending = __ballot_sync(kFull, !kempty(feas));
+__device__ __forceinline__ bool mmw_prunes(const K S, const bool extendable, const K* __restrict__ sAdj, const int n,
+                                           const int k, const int lane) {
+  unsigned pending = __ballot_sync(kFull, extendable);
+  bool mine = false;
   while (pending) {
     const int j = __ffs(pending) - 1;
     pending &= pending - 1;
     const bool prune = mmw_exceeds<K>(kshfl(S, j), sAdj, n, k, lane);
-    if (prune && lane == j) feas = kzero<K>();
+    if (prune && lane == j) mine = true;
   }
-  return feas;
+  return mine;
 }
 
-// Keeps the feasible extensions v of S whose new set S u {v} hashes into
-// range `range` of `ranges` equal ranges of the hash space (the same split as
-// the home slot: the high word of hash * ranges).
+// One warp's scratch in shared memory: the 32 states of its chunk, the
+// component of each state's lowest vertex with its boundary, the queue of
+// (state, vertex) pairs (up to kTake of each state at a time), and the new sets
+// that wait for a place in the output list.
+constexpr int kTake = 16;
+constexpr int kStage = 256;
 template <class K>
-__device__ __forceinline__ K in_hash_range(const K S, K feas, const unsigned long long ranges,
-                                           const unsigned long long range) {
-  K keep = kzero<K>();
-  while (!kempty(feas)) {
-    const K vb = klsb(feas);
-    feas ^= vb;
-    if (__umul64hi(khash(S | vb), ranges) == range) keep |= vb;
-  }
-  return keep;
-}
+struct WarpScratch {
+  K state[32], comp[32], bnd[32];
+  K stage_key[kStage];
+  uint32_t stage_from[kStage];  // added vertex, or the parent's index (kParent)
+  uint16_t queue[32 * kTake];
+};
 
-// Packs the feasible (S, v) pairs of the warp's 32 states into the warp's
-// queue (entry = lane << 8 | v) and stores each lane's S; returns the number
-// of pairs (warp uniform).
+// Packs up to kTake (S, v) pairs of each of the warp's 32 states into the
+// warp's queue (entry = lane << 8 | v) and takes them out of c; returns the
+// number of pairs (warp uniform).  The pairs that need no search come first, so
+// that the searches run in as few rounds of the warp as they fill (a round
+// takes as long as its longest search).
 template <class K>
-__device__ __forceinline__ int build_queue(const K S, K feas, const int lane, K* __restrict__ sS,
-                                           uint16_t* __restrict__ sQ) {
-  const int cnt = kpopc(feas);
+__device__ __forceinline__ int build_queue(Candidates<K>& c, const int lane, WarpScratch<K>& w) {
+  const int n0 = min(kpopc(c.done), kTake);
+  const int n1 = min(kpopc(c.search), kTake - n0);
+  const int cnt = n0 | (n1 << 16);
   int incl = cnt;
 #pragma unroll
   for (int d = 1; d < 32; d <<= 1) {
@@ -356,15 +282,67 @@ __device__ __forceinline__ int build_queue(const K S, K feas, const int lane, K*
     if (lane >= d) incl += t;
   }
   const int total = __shfl_sync(kFull, incl, 31);
-  int pos = incl - cnt;
-  sS[lane] = S;
-  while (!kempty(feas)) {
-    const int v = klowest(feas);
-    feas = kdrop_lowest(feas);
-    sQ[pos++] = (uint16_t)((lane << 8) | v);
+  const int excl = incl - cnt;
+  int pos = excl & 0xffff;
+  for (int end = pos + n0; pos < end; ++pos) {
+    const K vb = klsb(c.done);
+    c.done ^= vb;
+    w.queue[pos] = (uint16_t)((lane << 8) | kindex(vb));
+  }
+  pos = (total & 0xffff) + (excl >> 16);
+  for (int end = pos + n1; pos < end; ++pos) {
+    const K vb = klsb(c.search);
+    c.search ^= vb;
+    w.queue[pos] = (uint16_t)((lane << 8) | kindex(vb));
   }
   __syncwarp();
-  return total;
+  return (total & 0xffff) + (total >> 16);
+}
+template <class K>
+__device__ __forceinline__ bool any_left(const Candidates<K>& c) {
+  return !kempty(c.done | c.search);
+}
+
+// The search's first half for one chunk: the component of min(S) and the cheap
+// test; returns the surviving candidates of this lane's state.  Inactive lanes
+// pass active = false.
+template <class K, bool kCanonical, bool kMMW = false>
+__device__ __forceinline__ Candidates<K> start_chunk(const K S, const bool active, const K* __restrict__ sAdj,
+                                                     const K valid, const K allowed, const int n, const int k,
+                                                     const int lane, WarpScratch<K>& w) {
+  K comp0 = kzero<K>(), b0 = kzero<K>();
+  Candidates<K> c{kzero<K>(), kzero<K>()};
+  if (active) {
+    if (kCanonical) min_component<K>(S, sAdj, comp0, b0);
+    c = cheap_candidates<K, kCanonical>(S, comp0, b0, sAdj, valid, allowed, k);
+  }
+  if (kMMW && mmw_prunes<K>(S, any_left(c), sAdj, n, k, lane)) c = Candidates<K>{kzero<K>(), kzero<K>()};
+  w.state[lane] = S;
+  w.comp[lane] = comp0;
+  w.bnd[lane] = b0;
+  return c;
+}
+
+// Tests the queued pairs (pair per lane) and packs the feasible ones to the
+// front of the queue; returns their number (warp uniform).
+template <class K>
+__device__ __forceinline__ int keep_feasible(WarpScratch<K>& w, const int total, const int lane,
+                                             const K* __restrict__ sAdj, const int k) {
+  int kept = 0;
+  for (int base = 0; base < total; base += 32) {
+    const int j = base + lane;
+    uint16_t e = 0;
+    bool ok = false;
+    if (j < total) {
+      e = w.queue[j];
+      ok = extension_feasible<K>(w.state[e >> 8], w.comp[e >> 8], w.bnd[e >> 8], e & 0xff, sAdj, k);
+    }
+    const unsigned m = __ballot_sync(kFull, ok);  // (every lane has read its entry)
+    if (ok) w.queue[kept + __popc(m & ((1u << lane) - 1u))] = e;
+    kept += __popc(m);
+    __syncwarp();
+  }
+  return kept;
 }
 
 // Where the winners of the inserts go.  With kParent the output records the
@@ -381,111 +359,169 @@ struct LevelOut {
   unsigned int* overflow;  // bit 0: output full, bit 1: probe limit
 };
 
-// Inserts the queued pairs into the table, U per lane at a
-// time: the first probe of every pair is issued before any result is
-// inspected, so each lane has several compare-and-swaps in flight.  Linear
-// probing from the home slot, at most max_probes slots.  Winners append
-// (S u {v}, pred or parent) with one atomic add per round of the warp.
-//
-// With kRanged the table is the slice of one hash range (in_hash_range): the
-// home slot spreads the range's hashes over the slice (the high word of
-// (hash * ranges mod 2^64) * slots), no predecessor is stored, and output
-// positions from split on go to tail[position - split] when tail is given (a
-// list continued in a second buffer).
-template <class K, bool kParent, int U = TW_INSERT_UNROLL, bool kRanged = false>
-__device__ __forceinline__ void insert_queue(const uint16_t* __restrict__ sQ, const K* __restrict__ sS,
-                                             const int total, const int lane, K* __restrict__ table,
-                                             const unsigned long long slots, const int max_probes,
-                                             const LevelOut<K, kParent>& out, const unsigned long long ranges = 1,
-                                             K* tail = nullptr, const unsigned long long split = 0) {
-  const K empty = kones<K>();
-  const unsigned lanemask_lt = (1u << lane) - 1u;
-  for (int base = 0; base < total; base += 32 * U) {
-    K key[U];
-    int vv[U];
-    int src[U];
-    unsigned long long h[U];
-    int st[U];  // 0 idle, 1 probing, 2 inserted, 3 already present or given up
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      const int j = base + u * 32 + lane;
-      st[u] = 0;
-      vv[u] = 0;
-      src[u] = 0;
-      h[u] = 0;
-      key[u] = kzero<K>();
-      if (j < total) {
-        const uint16_t e = sQ[j];
-        vv[u] = e & 0xff;
-        src[u] = e >> 8;
-        key[u] = sS[src[u]] | kbit<K>(vv[u]);
-        h[u] = kRanged ? home_slot(khash(key[u]) * ranges, slots) : home_slot(khash(key[u]), slots);
-        st[u] = 1;
-      }
-    }
-    K old[U];
-#pragma unroll
-    for (int u = 0; u < U; ++u)
-      if (st[u] == 1) old[u] = kcas(&table[h[u]], empty, key[u]);
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      if (st[u] != 1) continue;
-      if (old[u] == empty) {
-        st[u] = 2;
-      } else if (old[u] == key[u]) {
-        st[u] = 3;
-      } else {
-        for (int probe = 1;; ++probe) {
-          if (probe >= max_probes) {
-            atomicOr(out.overflow, 2u);
-            st[u] = 3;
-            break;
-          }
-          h[u] = (h[u] + 1ull == slots) ? 0ull : h[u] + 1ull;
-          const K o = kcas(&table[h[u]], empty, key[u]);
-          if (o == empty) {
-            st[u] = 2;
-            break;
-          }
-          if (o == key[u]) {
-            st[u] = 3;
-            break;
-          }
-        }
-      }
-    }
-    unsigned wm[U];
-    int wins = 0;
-#pragma unroll
-    for (int u = 0; u < U; ++u) {
-      wm[u] = __ballot_sync(kFull, st[u] == 2);
-      wins += __popc(wm[u]);
-    }
-    if (wins) {
-      unsigned long long b = 0;
-      if (lane == 0) b = atomicAdd(out.count, (unsigned long long)wins);
-      b = __shfl_sync(kFull, b, 0);
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        if (st[u] == 2) {
-          const unsigned long long o = b + (unsigned long long)__popc(wm[u] & lanemask_lt);
-          if (o < out.cap) {
-            if (kRanged && tail != nullptr && o >= split)
-              kstore_cs(&tail[o - split], key[u]);
-            else
-              kstore_cs(&out.keys[o], key[u]);
-            if (kParent)
-              __stcs(&out.parent[o], out.parent_base + (uint32_t)src[u]);
-            else if (!kRanged)
-              __stcs(reinterpret_cast<signed char*>(&out.pred[o]), (signed char)vv[u]);
-          } else {
-            atomicOr(out.overflow, 1u);
-          }
-        }
-        b += (unsigned long long)__popc(wm[u]);
-      }
+// Moves the warp's staged new sets to the output list: one atomic add for all of
+// them.  (Every add of a level goes to the same counter, which takes about one
+// in 2.6 ns; with one add per 64 pairs that was the whole time of a level, with
+// one per 200 new sets it no longer shows.)  With kRanged no predecessor is
+// stored and output positions from split on go to tail[position - split] when
+// tail is given (a list continued in a second buffer).
+template <class K, bool kParent, bool kRanged>
+__device__ __forceinline__ void flush_stage(WarpScratch<K>& w, int& staged, const int lane,
+                                            const LevelOut<K, kParent>& out, K* tail, const unsigned long long split) {
+  if (staged == 0) return;
+  __syncwarp();
+  unsigned long long b = 0;
+  if (lane == 0) b = atomicAdd(out.count, (unsigned long long)staged);
+  b = __shfl_sync(kFull, b, 0);
+  for (int j = lane; j < staged; j += 32) {
+    const unsigned long long o = b + (unsigned long long)j;
+    if (o < out.cap) {
+      if (kRanged && tail != nullptr && o >= split)
+        kstore_cs(&tail[o - split], w.stage_key[j]);
+      else
+        kstore_cs(&out.keys[o], w.stage_key[j]);
+      if (kParent)
+        __stcs(&out.parent[o], w.stage_from[j]);
+      else if (!kRanged)
+        __stcs(reinterpret_cast<signed char*>(&out.pred[o]), (signed char)w.stage_from[j]);
+    } else {
+      atomicOr(out.overflow, 1u);
     }
   }
+  staged = 0;
+  __syncwarp();
+}
+
+// Slot of the sector in which key stands or may be put: the first of its slots
+// from `from` on that may be empty, kPresent when key comes before that, kFull
+// when every slot holds another key.
+constexpr int kSlotPresent = -1, kSlotNone = -2;
+template <class K>
+__device__ __forceinline__ int find_slot(const Sector<K>& s, const K key, const int from) {
+  int pos = kSlotNone;
+#pragma unroll
+  for (int i = Sector<K>::kSlots - 1; i >= 0; --i) {
+    if (i < from) break;
+    if (s.x[i] == key)
+      pos = kSlotPresent;
+    else if (kmaybe_empty(s.x[i]))
+      pos = i;
+  }
+  return pos;
+}
+
+// Inserts key into the table from the first slot of sector b on; true when this
+// thread put it in, false when it was there or the probe limit was reached
+// (*overflow then gets bit 1).
+//
+// The table is probed in 32-byte sectors (4, 8 or 2 slots for 64-, 32- and
+// 128-bit keys): a key's home is the first slot of a sector, and probing goes on
+// slot by slot.  One load of the whole sector shows whether the key is there
+// (two of three pairs on the geometric n=40 graph) or where the first empty slot
+// is, so a pair costs one load and a new set one compare-and-swap more; only
+// full sectors and lost races take further round trips.  (Probing slot by slot
+// with compare-and-swaps took 16 of them per chunk of 32 states, most for a few
+// lanes and one after the other.)  Keys fill a sector from its front: a thread
+// tries a slot only after it saw the earlier ones hold other keys, so two
+// threads with the same key meet at the same slot.
+template <class K>
+__device__ __forceinline__ bool insert_key(K* __restrict__ table, const unsigned int sectors, const int max_sectors,
+                                           unsigned int b, const K key, unsigned int* overflow) {
+  constexpr int B = Sector<K>::kSlots;
+  const K empty = kones<K>();
+  K* at = table + (size_t)b * B;
+  Sector<K> s;
+  kload_sector(at, s);
+  int pos = find_slot<K>(s, key, 0);
+  if (pos == kSlotPresent) return false;
+  if (pos >= 0) {
+    const K o = kcas(at + pos, empty, key);
+    if (o == empty) return true;
+    if (o == key) return false;
+  }
+  // a full sector or a lost race (apart from the first probe: one loop for both
+  // made the kernel 6 to 23% slower)
+  int from = pos >= 0 ? pos + 1 : B;
+  for (int looked = 1;;) {
+    if (from >= B) {
+      if (++looked > max_sectors) {
+        atomicOr(overflow, 2u);
+        return false;
+      }
+      b = b + 1u == sectors ? 0u : b + 1u;
+      at = table + (size_t)b * B;
+      from = 0;
+    }
+    kload_sector(at, s);
+    pos = find_slot<K>(s, key, from);
+    if (pos == kSlotPresent) return false;
+    if (pos == kSlotNone) {
+      from = B;
+      continue;
+    }
+    const K o = kcas(at + pos, empty, key);
+    if (o == empty) return true;
+    if (o == key) return false;
+    from = pos + 1;
+  }
+}
+
+// Tests the queued pairs (pair per lane) and inserts the feasible ones into the
+// table; returns this lane's count of feasible pairs.
+//
+// One pair per lane at a time: with two in flight the kernel is 4% slower on the
+// geometric n=40 graph (9.40 against 9.05 ms of expand time), with three 9%
+// (more registers and code against latency that the other warps hide).
+// Winners are staged in shared memory (staged of them wait) and flushed when
+// the next round might not fit.
+//
+// With kRanged only the pairs whose new set hashes into range `range` of
+// `ranges` equal ranges of the hash space are inserted (all feasible ones are
+// pairs of one of the ranges); the table is the slice of that range (the home
+// spreads the range's hashes over the slice: the high word of (hash * ranges
+// mod 2^64) * sectors).
+template <class K, bool kParent, bool kRanged = false>
+__device__ __forceinline__ int search_insert(WarpScratch<K>& w, const int total, int& staged, const int lane,
+                                             const K* __restrict__ sAdj, const int k, K* __restrict__ table,
+                                             const unsigned long long slots, const int max_probes,
+                                             const LevelOut<K, kParent>& out, const unsigned long long ranges = 1,
+                                             const unsigned long long range = 0, K* tail = nullptr,
+                                             const unsigned long long split = 0) {
+  constexpr int B = Sector<K>::kSlots;
+  // (the 2^32 - 1 sectors that an index holds are 128 GB)
+  const unsigned int sectors = (unsigned int)min(slots / B, 0xffffffffull);
+  const int max_sectors = (max_probes + B - 1) / B;
+  int generated = 0;
+  for (int base = 0; base < total; base += 32) {
+    const bool have = base + lane < total;
+    const int e = have ? w.queue[base + lane] : 0;
+    const K S = w.state[e >> 8];
+    const K key = S | kbit<K>(e & 0xff);
+    bool ok = have && extension_feasible<K>(S, w.comp[e >> 8], w.bnd[e >> 8], e & 0xff, sAdj, k);
+    unsigned int home;
+    if (kRanged) {
+      const unsigned long long hash = khash(key);
+      ok = ok && __umul64hi(hash, ranges) == range;
+      home = (unsigned int)home_slot(hash * ranges, sectors);
+    } else {
+      home = __umulhi(khash32(key), sectors);
+    }
+    generated += ok ? 1 : 0;
+    // the lanes whose searches took longer are waited for here, so that the warp
+    // probes the table together
+    __syncwarp();
+    const bool won = ok && insert_key<K>(table, sectors, max_sectors, home, key, out.overflow);
+    __syncwarp();
+    if (staged > kStage - 32) flush_stage<K, kParent, kRanged>(w, staged, lane, out, tail, split);
+    const unsigned wm = __ballot_sync(kFull, won);
+    if (won) {
+      const int o = staged + __popc(wm & ((1u << lane) - 1u));
+      w.stage_key[o] = key;
+      w.stage_from[o] = kParent ? out.parent_base + (uint32_t)(e >> 8) : (uint32_t)(e & 0xff);
+    }
+    staged += __popc(wm);
+  }
+  return generated;
 }
 
 // A key from two 64-bit words (low word first).
@@ -562,11 +598,17 @@ __device__ __forceinline__ void plan_level(unsigned long long cnt, unsigned long
   *slots = max(64ull, (*table_est * 100ull + (unsigned long long)load_pct - 1ull) / (unsigned long long)load_pct);
 }
 
+// Adds the lanes' counts and, in lane 0, adds the sum to *total.
+__device__ __forceinline__ void add_warp_count(unsigned long long count, const int lane, unsigned long long* total) {
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) count += __shfl_xor_sync(kFull, count, d);
+  if (lane == 0 && count) atomicAdd(total, count);
+}
+
 // One level i -> i+1 by the whole block: the adjacency rows go to shared
 // memory, then each warp takes chunks of 32 consecutive states (coalesced key
-// loads), finds their feasible extensions (thread per state), queues the
-// pairs and inserts them cooperatively.  sState holds kWarps x 32 keys,
-// sQueue kWarps x 32 x kBits entries.
+// loads), queues their candidate pairs (thread per state), and tests and
+// inserts the pairs (pair per lane).  scratch holds one entry per warp.
 //
 // With kBlockLocal the block expands the whole level alone (its warps take the
 // chunks in turn): a persistent kernel whose blocks work on different graphs.
@@ -575,20 +617,19 @@ __device__ __forceinline__ void plan_level(unsigned long long cnt, unsigned long
 // With kGroup the level is expanded by a group of the grid's blocks (block
 // group_block of group_blocks) instead of the whole grid.  Ranged kernels may
 // continue the output list in out_tail from position out_split on.
-template <class K, int kWarps, int U = TW_INSERT_UNROLL, bool kMMW = false, bool kRanged = false,
+template <class K, int kWarps, bool kMMW = false, bool kRanged = false,
           bool kBlockLocal = false, bool kKeysL2 = false, bool kGroup = false>
-__device__ __forceinline__ void expand_level(const ExpandParams<K>& p, K* sAdj, K* sState, uint16_t* sQueue,
+__device__ __forceinline__ void expand_level(const ExpandParams<K>& p, K* sAdj, WarpScratch<K>* scratch,
                                              const unsigned group_block = 0, const unsigned group_blocks = 0,
                                              K* out_tail = nullptr, const unsigned long long out_split = 0) {
-  constexpr int kBits = KeyTraits<K>::kBits;
   for (int i = threadIdx.x; i < p.n; i += blockDim.x) sAdj[i] = p.adj[i];
   __syncthreads();
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
-  K* sS = sState + warp * 32;
-  uint16_t* sQ = sQueue + warp * 32 * kBits;
+  WarpScratch<K>& w = scratch[warp];
   const K valid = kfirst_n<K>(p.n);
-  unsigned long long generated_total = 0;
+  unsigned long long generated = 0;
+  int staged = 0;
   const unsigned long long n_chunks = (p.n_in + 31ull) / 32ull;
   const unsigned long long blk = kGroup ? (unsigned long long)group_block : (unsigned long long)blockIdx.x;
   const unsigned long long nblk = kGroup ? (unsigned long long)group_blocks : (unsigned long long)gridDim.x;
@@ -608,16 +649,17 @@ __device__ __forceinline__ void expand_level(const ExpandParams<K>& p, K* sAdj, 
     const K S = active ? (kKeysL2 ? kload_cg(&p.in_keys[idx]) : kload_cs(&p.in_keys[idx])) : valid;
     // (minor-min-width pruning drops some parents, so it extends by every
     // feasible vertex)
-    K feas = active ? feasible_extensions<K, !kMMW>(S, sAdj, valid, p.allowed, p.k) : kzero<K>();
-    if (kMMW) feas = mmw_filter<K>(S, feas, sAdj, p.n, p.k, lane);
-    if (kRanged) feas = in_hash_range<K>(S, feas, p.ranges, p.range);
-    const int total = build_queue<K>(S, feas, lane, sS, sQ);
-    generated_total += (unsigned long long)total;
-    insert_queue<K, false, U, kRanged>(sQ, sS, total, lane, p.table, p.table_slots, p.max_probes, out, p.ranges,
-                                       out_tail, out_split);
-    __syncwarp();
+    Candidates<K> c = start_chunk<K, !kMMW, kMMW>(S, active, sAdj, valid, p.allowed, p.n, p.k, lane, w);
+    do {
+      const int total = build_queue<K>(c, lane, w);
+      generated += (unsigned long long)search_insert<K, false, kRanged>(w, total, staged, lane, sAdj, p.k, p.table,
+                                                                           p.table_slots, p.max_probes, out, p.ranges,
+                                                                           p.range, out_tail, out_split);
+      __syncwarp();
+    } while (__any_sync(kFull, any_left(c)));
   }
-  if (lane == 0 && generated_total) atomicAdd(&p.ctr->generated, generated_total);
+  flush_stage<K, false, kRanged>(w, staged, lane, out, out_tail, out_split);
+  add_warp_count(generated, lane, &p.ctr->generated);
 }
 
 // The backward walk by one block: from the first set of level `last`, find

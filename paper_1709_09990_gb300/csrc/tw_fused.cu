@@ -117,7 +117,7 @@ struct FusedArgs {
 // gave up); *last = index of the final level built.
 template <class K>
 __device__ int group_decide(const FusedArgs<K>& a, int grp, unsigned int gb, unsigned int nb, int k,
-                            unsigned long long dirty[2], int* last, K* sAdj, K* sState, uint16_t* sQueue) {
+                            unsigned long long dirty[2], int* last, K* sAdj, core::WarpScratch<K>* sScratch) {
   FusedState* st = a.st[grp];
   unsigned int* error = &a.st[0]->error;
   K* keys = a.keys[grp];
@@ -172,8 +172,7 @@ __device__ int group_decide(const FusedArgs<K>& a, int grp, unsigned int gb, uns
     unsigned long long got = 0;
     for (int attempt = 0;; ++attempt) {
       p.table_slots = slots;
-      core::expand_level<K, kFusedWarps, TW_INSERT_UNROLL, false, false, false, true, true>(p, sAdj, sState,
-                                                                                           sQueue, gb, nb);
+      core::expand_level<K, kFusedWarps, false, false, false, true, true>(p, sAdj, sScratch, gb, nb);
       // meanwhile empty the table the previous level used
       for (unsigned long long j = gtid; j < dirty[1 - t]; j += gthreads) a.table[grp][1 - t][j] = kones<K>();
       dirty[1 - t] = 0;
@@ -221,10 +220,8 @@ __device__ int group_decide(const FusedArgs<K>& a, int grp, unsigned int gb, uns
 template <class K>
 __global__ void __launch_bounds__(kFusedWarps * 32, ResidentWarps<K>::value / kFusedWarps)
     fused_solve_kernel(const FusedArgs<K> a) {
-  constexpr int kBits = KeyTraits<K>::kBits;
-  __shared__ K sAdj[kBits];
-  __shared__ K sState[kFusedWarps * 32];
-  __shared__ uint16_t sQueue[kFusedWarps * 32 * kBits];
+  __shared__ K sAdj[KeyTraits<K>::kBits];
+  __shared__ core::WarpScratch<K> sScratch[kFusedWarps];
   __shared__ K128 sTdAdj[128];
   __shared__ int sPos[128];
   __shared__ K sWalk;
@@ -245,7 +242,7 @@ __global__ void __launch_bounds__(kFusedWarps * 32, ResidentWarps<K>::value / kF
       const int k = k_base + grp;
       int result = -1, last = 0;
       if (k <= a.k_last) {
-        result = group_decide<K>(a, grp, gb, nb, k, dirty, &last, sAdj, sState, sQueue);
+        result = group_decide<K>(a, grp, gb, nb, k, dirty, &last, sAdj, sScratch);
         if (result == -2) return;
       }
       if (gb == 0 && threadIdx.x == 0) {

@@ -92,10 +92,8 @@ __global__ void graph_clear_kernel(const GraphState* __restrict__ st, uint4* __r
 template <class K, int kWarps, bool kMMW>
 __global__ void __launch_bounds__(kWarps * 32, ResidentWarps<K>::value / kWarps)
     graph_expand_kernel(const GraphState* __restrict__ st, const ExpandParams<K> base) {
-  constexpr int kBits = KeyTraits<K>::kBits;
-  __shared__ K sAdj[kBits];
-  __shared__ K sState[kWarps * 32];
-  __shared__ uint16_t sQueue[kWarps * 32 * kBits];
+  __shared__ K sAdj[KeyTraits<K>::kBits];
+  __shared__ core::WarpScratch<K> sScratch[kWarps];
   if (st->done || st->bail) return;
   ExpandParams<K> p = base;
   const int cur = st->cur;
@@ -105,7 +103,7 @@ __global__ void __launch_bounds__(kWarps * 32, ResidentWarps<K>::value / kWarps)
   p.out_pred = base.out_pred + st->out_off;
   p.out_cap = st->out_cap;
   p.table_slots = st->table_slots;
-  core::expand_level<K, kWarps, TW_INSERT_UNROLL, kMMW>(p, sAdj, sState, sQueue);
+  core::expand_level<K, kWarps, kMMW>(p, sAdj, sScratch);
 }
 
 int sm_count() {

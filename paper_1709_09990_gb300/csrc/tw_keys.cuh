@@ -126,6 +126,27 @@ __device__ __forceinline__ unsigned long long khash(uint32_t a) { return fmix64(
 __device__ __forceinline__ unsigned long long khash(unsigned long long a) { return fmix64(a); }
 __device__ __forceinline__ unsigned long long khash(K128 a) { return fmix64(a.lo ^ fmix64(a.hi ^ 0x9e3779b97f4a7c15ull)); }
 
+// A 32-bit hash for the home of a key in the table of one level: the words of the
+// key times odd constants, folded and mixed twice by multiply and xor-shift (a
+// third of the instructions of khash; its value is no result, it only spreads
+// the keys).
+__device__ __forceinline__ unsigned int mix32(unsigned int x) {
+  x ^= x >> 16;
+  x *= 0x9e3779b1u;
+  x ^= x >> 15;
+  x *= 0xbb67ae85u;
+  return x ^ (x >> 13);
+}
+__device__ __forceinline__ unsigned int khash32(uint32_t a) { return mix32(a * 0x3c6ef373u); }
+__device__ __forceinline__ unsigned int khash32(unsigned long long a) {
+  const unsigned long long m = (unsigned long long)(unsigned int)a * 0x6a09e667f3bcc909ull +
+                               (unsigned long long)(unsigned int)(a >> 32) * 0xbb67ae8584caa73bull;
+  return mix32((unsigned int)m ^ (unsigned int)(m >> 32));
+}
+__device__ __forceinline__ unsigned int khash32(K128 a) {
+  return mix32(khash32(a.lo) + 0x510e527fu * khash32(a.hi ^ 0x3c6ef372fe94f82bull));
+}
+
 // Level fingerprint fp(S) = mix(w0 ^ mix(w1)) with mix the splitmix64 output
 // function (Steele, Lea & Flood 2014).  Order independent once summed.
 __device__ __forceinline__ unsigned long long splitmix_out(unsigned long long z) {
@@ -160,6 +181,39 @@ __device__ __forceinline__ K128 kcas(K128* p, K128 cmp, K128 val) {
       : "memory");
   return old;
 }
+
+// One 32-byte sector of a hash table, read with one access that goes to the L2
+// (other SMs write the table during a level).  Words are read whole; the two
+// halves of a 128-bit key may be of different times.
+template <class K> struct Sector { static constexpr int kSlots = 32 / (int)sizeof(K); K x[kSlots]; };
+__device__ __forceinline__ void kload_sector(const uint32_t* p, Sector<uint32_t>& s) {
+  asm volatile("ld.relaxed.gpu.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
+               : "=r"(s.x[0]), "=r"(s.x[1]), "=r"(s.x[2]), "=r"(s.x[3]), "=r"(s.x[4]), "=r"(s.x[5]), "=r"(s.x[6]),
+                 "=r"(s.x[7])
+               : "l"(p)
+               : "memory");
+}
+__device__ __forceinline__ void kload_sector(const unsigned long long* p, Sector<unsigned long long>& s) {
+  asm volatile("ld.relaxed.gpu.global.v4.b64 {%0, %1, %2, %3}, [%4];"
+               : "=l"(s.x[0]), "=l"(s.x[1]), "=l"(s.x[2]), "=l"(s.x[3])
+               : "l"(p)
+               : "memory");
+}
+__device__ __forceinline__ void kload_sector(const K128* p, Sector<K128>& s) {
+  unsigned long long a, b, c, d;
+  asm volatile("ld.relaxed.gpu.global.v4.b64 {%0, %1, %2, %3}, [%4];"
+               : "=l"(a), "=l"(b), "=l"(c), "=l"(d)
+               : "l"(p)
+               : "memory");
+  s.x[0] = K128{a, b};
+  s.x[1] = K128{c, d};
+}
+
+// May the slot that was read as x be empty?  (A 128-bit slot whose halves were
+// read around a write counts as maybe empty: its compare-and-swap tells.)
+__device__ __forceinline__ bool kmaybe_empty(uint32_t x) { return x == ~0u; }
+__device__ __forceinline__ bool kmaybe_empty(unsigned long long x) { return x == ~0ull; }
+__device__ __forceinline__ bool kmaybe_empty(K128 x) { return x.lo == ~0ull || x.hi == ~0ull; }
 
 // Load that bypasses L1 (the table is written by other SMs during a level).
 __device__ __forceinline__ uint32_t kload_cg(const uint32_t* p) { return __ldcg(p); }

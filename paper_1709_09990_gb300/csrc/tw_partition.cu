@@ -86,10 +86,8 @@ __global__ void __launch_bounds__(kWarps * 32, 6)
     emit_kernel(const ExpandParams<K> p, int P, K* __restrict__ cand_key, uint8_t* __restrict__ cand_v,
                 unsigned long long region_cap, unsigned long long* __restrict__ region_cnt,
                 unsigned int* __restrict__ overflow) {
-  constexpr int kBits = KeyTraits<K>::kBits;
-  __shared__ K sAdj[kBits];
-  __shared__ K sState[kWarps * 32];
-  __shared__ uint16_t sQueue[kWarps * 32 * kBits];
+  __shared__ K sAdj[KeyTraits<K>::kBits];
+  __shared__ core::WarpScratch<K> sScratch[kWarps];
   __shared__ int sTotal[kWarps];
   __shared__ int sHist[kMaxRanges];
   __shared__ int sCursor[kMaxRanges];
@@ -105,48 +103,51 @@ __global__ void __launch_bounds__(kWarps * 32, 6)
     const unsigned long long idx = b * (kWarps * 32) + warp * 32 + lane;
     const bool active = idx < p.n_in;
     const K S = active ? p.in_keys[idx] : valid;
-    K feas = active ? core::feasible_extensions<K>(S, sAdj, valid, p.allowed, p.k) : kzero<K>();
-    if (p.mmw) feas = core::mmw_filter<K>(S, feas, sAdj, p.n, p.k, lane);
-    const int total = core::build_queue<K>(S, feas, lane, sState + warp * 32, sQueue + warp * 32 * kBits);
-    if (lane == 0) sTotal[warp] = total;
-    for (int r = threadIdx.x; r < P; r += blockDim.x) sHist[r] = 0;
-    __syncthreads();
-    int start[kWarps + 1];
-    start[0] = 0;
-#pragma unroll
-    for (int w = 0; w < kWarps; ++w) start[w + 1] = start[w] + sTotal[w];
-    const int T = start[kWarps];
-    generated_total += (unsigned long long)(threadIdx.x == 0 ? T : 0);
-    // histogram of the block's pairs over the ranges
-    for (int e = threadIdx.x; e < T; e += blockDim.x) {
-      int w = 0;
-      while (e >= start[w + 1]) ++w;
-      const uint16_t q = sQueue[w * 32 * kBits + (e - start[w])];
-      const K key = sState[w * 32 + (q >> 8)] | kbit<K>(q & 0xff);
-      atomicAdd(&sHist[range_of(khash(key), P)], 1);
-    }
-    __syncthreads();
-    for (int r = threadIdx.x; r < P; r += blockDim.x) {
-      sCursor[r] = 0;
-      sBase[r] = sHist[r] ? atomicAdd(&region_cnt[r], (unsigned long long)sHist[r]) : 0ull;
-    }
-    __syncthreads();
-    // scatter: the block's pairs of one range land next to each other
-    for (int e = threadIdx.x; e < T; e += blockDim.x) {
-      int w = 0;
-      while (e >= start[w + 1]) ++w;
-      const uint16_t q = sQueue[w * 32 * kBits + (e - start[w])];
-      const K key = sState[w * 32 + (q >> 8)] | kbit<K>(q & 0xff);
-      const int r = range_of(khash(key), P);
-      const unsigned long long pos = sBase[r] + (unsigned long long)atomicAdd(&sCursor[r], 1);
-      if (pos < region_cap) {
-        store_stream(&cand_key[(unsigned long long)r * region_cap + pos], key);
-        store_stream(&cand_v[(unsigned long long)r * region_cap + pos], (uint8_t)(q & 0xff));
-      } else {
-        atomicOr(overflow, 1u);
+    core::WarpScratch<K>& ws = sScratch[warp];
+    core::Candidates<K> c =
+        p.mmw ? core::start_chunk<K, false, true>(S, active, sAdj, valid, p.allowed, p.n, p.k, lane, ws)
+              : core::start_chunk<K, true>(S, active, sAdj, valid, p.allowed, p.n, p.k, lane, ws);
+    do {
+      const int total = core::keep_feasible<K>(ws, core::build_queue<K>(c, lane, ws), lane, sAdj, p.k);
+      if (lane == 0) sTotal[warp] = total;
+      for (int r = threadIdx.x; r < P; r += blockDim.x) sHist[r] = 0;
+      __syncthreads();
+      int start[kWarps + 1];
+      start[0] = 0;
+  #pragma unroll
+      for (int w = 0; w < kWarps; ++w) start[w + 1] = start[w] + sTotal[w];
+      const int T = start[kWarps];
+      generated_total += (unsigned long long)(threadIdx.x == 0 ? T : 0);
+      // histogram of the block's pairs over the ranges
+      for (int e = threadIdx.x; e < T; e += blockDim.x) {
+        int w = 0;
+        while (e >= start[w + 1]) ++w;
+        const uint16_t q = sScratch[w].queue[e - start[w]];
+        const K key = sScratch[w].state[q >> 8] | kbit<K>(q & 0xff);
+        atomicAdd(&sHist[range_of(khash(key), P)], 1);
       }
-    }
-    __syncthreads();
+      __syncthreads();
+      for (int r = threadIdx.x; r < P; r += blockDim.x) {
+        sCursor[r] = 0;
+        sBase[r] = sHist[r] ? atomicAdd(&region_cnt[r], (unsigned long long)sHist[r]) : 0ull;
+      }
+      __syncthreads();
+      // scatter: the block's pairs of one range land next to each other
+      for (int e = threadIdx.x; e < T; e += blockDim.x) {
+        int w = 0;
+        while (e >= start[w + 1]) ++w;
+        const uint16_t q = sScratch[w].queue[e - start[w]];
+        const K key = sScratch[w].state[q >> 8] | kbit<K>(q & 0xff);
+        const int r = range_of(khash(key), P);
+        const unsigned long long pos = sBase[r] + (unsigned long long)atomicAdd(&sCursor[r], 1);
+        if (pos < region_cap) {
+          store_stream(&cand_key[(unsigned long long)r * region_cap + pos], key);
+          store_stream(&cand_v[(unsigned long long)r * region_cap + pos], (uint8_t)(q & 0xff));
+        } else {
+          atomicOr(overflow, 1u);
+        }
+      }
+    } while (__syncthreads_or(core::any_left(c)));
   }
   if (threadIdx.x == 0 && generated_total) atomicAdd(&p.ctr->generated, generated_total);
 }
