@@ -24,6 +24,15 @@ constexpr double kEvictStates = double(1 << 21);
 constexpr unsigned long long kStepSlots = 1ull << 27;   // table slots per step
 constexpr unsigned long long kStepOut = 1ull << 26;     // output states per step
 constexpr int kBatchProbes = 256;
+// States that one block of copy_segments_kernel moves: levels are copied in
+// pieces of this size, so that a level of a million sets takes the whole GPU
+// and not one block (the copies of a 512-graph batch took 137 of its 371 ms).
+constexpr unsigned long long kCopyPiece = 8192;
+
+void add_copy(std::vector<CopySeg>* list, unsigned long long src, unsigned long long dst, unsigned long long count) {
+  for (unsigned long long at = 0; at < count; at += kCopyPiece)
+    list->push_back({src + at, dst + at, std::min(kCopyPiece, count - at)});
+}
 
 struct BGraph {
   int in_idx = 0;
@@ -121,7 +130,7 @@ struct BatchRun {
     for (BGraph& x : g) {
       if (x.state != 0) continue;
       for (LevelRec& l : x.levels) {
-        if (l.count) cs.push_back({l.off, top, l.count});
+        add_copy(&cs, l.off, top, l.count);
         l.off = top;
         top += l.count;
       }
@@ -180,11 +189,13 @@ bool record_answer(BGraph& x, bool yes) {
 }
 
 // The batched part: every graph of idx either finishes here (state 1) or is
-// returned in *evicted for the single-graph path.
+// returned in *evicted for the single-graph path.  known_no (by graph index, or
+// null): the largest k that is known to answer no, -1 for none; raised here
+// for the evicted graphs, so that their sweep goes on where it stopped.
 int run_batch(tw_ctx* c, const std::vector<HostGraph>& graphs, const std::vector<int>& idx,
               const std::vector<float>* hint, const std::vector<int64_t>& order_off, int* htw,
               std::vector<int32_t>* hord, std::vector<int>* hst, tw_stats* st, std::vector<int>* evicted,
-              const BatchDecide* dm) {
+              const BatchDecide* dm, std::vector<int>* known_no = nullptr) {
   BatchRun B(c);
   const int G = (int)idx.size();
   if (G == 0) return TW_OK;
@@ -220,6 +231,7 @@ int run_batch(tw_ctx* c, const std::vector<HostGraph>& graphs, const std::vector
       x.in_idx = idx[j];
       x.n = graphs[idx[j]].n;
       x.lb = std::max(b[4 * j], b[4 * j + 1]);
+      if (known_no) x.lb = std::max(x.lb, (*known_no)[idx[j]] + 1);
       x.no_max = x.lb - 1;
       int k0 = x.lb;
       if (hint) k0 = (int)std::lround((*hint)[idx[j]]);
@@ -231,8 +243,11 @@ int run_batch(tw_ctx* c, const std::vector<HostGraph>& graphs, const std::vector
   int64_t total_n = 0;
   for (int j = 0; j < G; ++j) total_n = std::max<int64_t>(total_n, B.g[j].order_off + B.g[j].n);
   if ((rc = dev_alloc(&B.orders, (size_t)total_n))) return rc;
+  // (a step's pieces: its segments' last ones and the whole ones of its output;
+  // grown below if a step ever has more)
+  size_t copy_room = (size_t)G + (size_t)(kStepOut / kCopyPiece) + 1024;
   if ((rc = dev_alloc(&B.segs, G)) || (rc = dev_alloc(&B.cbeg, (size_t)G + 1)) || (rc = dev_alloc(&B.ctr, G)) ||
-      (rc = dev_alloc(&B.copies, G)) || (rc = dev_alloc(&B.walks, G)) ||
+      (rc = dev_alloc(&B.copies, copy_room)) || (rc = dev_alloc(&B.walks, G)) ||
       (rc = dev_alloc(&B.lvl, (size_t)G * 65)))
     return rc;
   std::vector<BatchSeg> segs;
@@ -458,11 +473,18 @@ int run_batch(tw_ctx* c, const std::vector<HostGraph>& graphs, const std::vector
         st->candidates += segs[s2].in_count * (unsigned long long)(x.n - i);
         st->generated += h.generated;
       }
-      if (h.out_count) copies.push_back({segs[s2].o_off, B.atop, h.out_count});
+      add_copy(&copies, segs[s2].o_off, B.atop, h.out_count);
       x.levels.push_back({B.atop, h.out_count});
       B.atop += h.out_count;
     }
     if (!copies.empty()) {
+      if (copies.size() > copy_room) {
+        TW_CK(cudaStreamSynchronize(c->stream));
+        cudaFree(B.copies);
+        B.copies = nullptr;
+        copy_room = 2 * copies.size();
+        if ((rc = dev_alloc(&B.copies, copy_room))) return rc;
+      }
       TW_CK(cudaMemcpyAsync(B.copies, copies.data(), copies.size() * sizeof(CopySeg), cudaMemcpyHostToDevice,
                             c->stream));
       TW_LAUNCH(c, launch_copy_segments(B.copies, (int)copies.size(), B.okeys, B.opar, B.akeys, B.apar, c->stream));
@@ -484,7 +506,10 @@ int run_batch(tw_ctx* c, const std::vector<HostGraph>& graphs, const std::vector
       for (int v = 0; v < x.n; ++v) (*hord)[x.order_off + v] = dord[x.order_off + v];
   }
   for (BGraph& x : B.g)
-    if (x.state == 2) evicted->push_back(x.in_idx);
+    if (x.state == 2) {
+      evicted->push_back(x.in_idx);
+      if (known_no) (*known_no)[x.in_idx] = std::max((*known_no)[x.in_idx], x.no_max);
+    }
   return TW_OK;
 }
 
@@ -521,7 +546,7 @@ struct DevMem {
 int run_batch_persistent(tw_ctx* c, const std::vector<HostGraph>& graphs, const std::vector<int>& idx,
                          const std::vector<float>* hint, const std::vector<int64_t>& order_off, int* htw,
                          std::vector<int32_t>* hord, std::vector<int>* hst, tw_stats* st, std::vector<int>* evicted,
-                         const BatchDecide* dm, int warps);
+                         const BatchDecide* dm, int warps, std::vector<int>* known_no = nullptr);
 
 // With tw_config.autotune, the first batch of at least 512 graphs times the
 // persistent kernel with 4 and with 8 warps per block on a sample of 256 of
@@ -555,7 +580,7 @@ int batch_warps(tw_ctx* c, const std::vector<HostGraph>& graphs, const std::vect
 int run_batch_persistent(tw_ctx* c, const std::vector<HostGraph>& graphs, const std::vector<int>& idx,
                          const std::vector<float>* hint, const std::vector<int64_t>& order_off, int* htw,
                          std::vector<int32_t>* hord, std::vector<int>* hst, tw_stats* st, std::vector<int>* evicted,
-                         const BatchDecide* dm, int warps) {
+                         const BatchDecide* dm, int warps, std::vector<int>* known_no) {
   const int G = (int)idx.size();
   if (G == 0) return TW_OK;
   if (warps == 0) warps = batch_warps(c, graphs, idx, hint, order_off, dm);
@@ -689,6 +714,7 @@ int run_batch_persistent(tw_ctx* c, const std::vector<HostGraph>& graphs, const 
     const int gi = q[j];
     if (hst_p[j] != 0) {
       evicted->push_back(gi);
+      if (known_no && !dm) (*known_no)[gi] = std::max((*known_no)[gi], -1 - htw_p[j]);
       continue;
     }
     (*hst)[gi] = TW_OK;
@@ -720,14 +746,15 @@ int solve_batch_gpu(tw_ctx* c, const std::vector<HostGraph>& graphs, const std::
   NvtxRange range("tw solve_batch graphs=%d", (int)idx.size());
   std::vector<int> small, single;
   for (int i : idx) (graphs[i].n <= 64 ? small : single).push_back(i);
+  std::vector<int> known_no(graphs.size(), -1);  // decide runs answered no before a graph moved on
   int rc;
   if (c->cfg.batch_kernel == 1) {
-    rc = run_batch(c, graphs, small, hint, order_off, htw, hord, hst, st, &single, nullptr);
+    rc = run_batch(c, graphs, small, hint, order_off, htw, hord, hst, st, &single, nullptr, &known_no);
   } else {
     std::vector<int> outgrown;
-    rc = run_batch_persistent(c, graphs, small, hint, order_off, htw, hord, hst, st, &outgrown, nullptr, 0);
+    rc = run_batch_persistent(c, graphs, small, hint, order_off, htw, hord, hst, st, &outgrown, nullptr, 0, &known_no);
     if (rc == TW_OK && !outgrown.empty())
-      rc = run_batch(c, graphs, outgrown, hint, order_off, htw, hord, hst, st, &single, nullptr);
+      rc = run_batch(c, graphs, outgrown, hint, order_off, htw, hord, hst, st, &single, nullptr, &known_no);
   }
   if (rc) return rc;
   for (int gi : single) {
@@ -737,10 +764,13 @@ int solve_batch_gpu(tw_ctx* c, const std::vector<HostGraph>& graphs, const std::
     tw_stats local;
     std::memset(&local, 0, sizeof(local));
     if (hint) {
-      r2 = solve_hinted(c, hg, (*hint)[gi], &htw[gi], hord ? &ord : nullptr, &local);
+      r2 = solve_hinted(c, hg, (*hint)[gi], &htw[gi], hord ? &ord : nullptr, &local, known_no[gi] + 1);
     } else {
+      // (a graph that left the batched kernels has levels beyond the fused
+      // solve's arena)
       ord.assign(hg.n, -1);
-      r2 = solve_graph(c, hg, &htw[gi], hord ? ord.data() : nullptr, nullptr, nullptr, &local, 0);
+      r2 = solve_graph(c, hg, &htw[gi], hord ? ord.data() : nullptr, nullptr, nullptr, &local, known_no[gi] + 1,
+                       hg.n > 64);
     }
     if (st && r2 == TW_OK) {
       st->states_expanded += local.states_expanded;

@@ -245,7 +245,7 @@ __global__ void __launch_bounds__(kWarps * 32, 24 / kWarps) batch_solve_kernel(c
     if (!ok) {
       if (threadIdx.x == 0) {
         a.status[g] = 2;
-        a.tw[g] = -1;
+        a.tw[g] = -1 - no_max;  // every k up to no_max answers no
       }
       __syncthreads();
       continue;

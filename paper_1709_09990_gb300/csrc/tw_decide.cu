@@ -1394,7 +1394,7 @@ int launch_lower_bounds(tw_ctx* c, const HostGraph& g, const int32_t** d_bounds)
 }
 
 int solve_graph(tw_ctx* c, const HostGraph& g, int* tw_out, int32_t* order, int32_t* td_parent, uint64_t* td_bags,
-                tw_stats* st, int k_first) {
+                tw_stats* st, int k_first, bool try_fused) {
   NvtxRange range("tw solve n=%d", g.n);
   Timer t;
   const unsigned long long launches0 = c->launches;
@@ -1414,7 +1414,7 @@ int solve_graph(tw_ctx* c, const HostGraph& g, int* tw_out, int32_t* order, int3
   int k0 = k_first;
   bool fused_done = false;
   bool have_bounds = false;
-  if (!c->cfg.ub_shortcut && fused_eligible(c, g)) {
+  if (!c->cfg.ub_shortcut && try_fused && fused_eligible(c, g)) {
     // the fused solve reads the lower bounds on the device: no host round
     // trip between the bounds and the sweep
     const int32_t* d_bounds = nullptr;
@@ -1440,7 +1440,7 @@ int solve_graph(tw_ctx* c, const HostGraph& g, int* tw_out, int32_t* order, int3
     if (c->cfg.ub_shortcut && lb == ub && !want_walk) {
       tw = ub;
       fused_done = true;  // (no decide run and no walk)
-    } else if (c->cfg.ub_shortcut && fused_eligible(c, g)) {
+    } else if (c->cfg.ub_shortcut && try_fused && fused_eligible(c, g)) {
       int status = 0, ans = -1, bail_k = -1;
       rc = run_fused(c, g, kc, k0, g.n - 1, &R, &status, &ans, &bail_k, st, nullptr);
       if (rc) return rc;
@@ -1494,13 +1494,13 @@ int solve_graph(tw_ctx* c, const HostGraph& g, int* tw_out, int32_t* order, int3
 // and no at tw-1 (or tw = lower bound) certify the answer.  Returns the
 // treewidth in *tw_out and the ordering of the yes run at tw in order_host.
 int solve_hinted(tw_ctx* c, const HostGraph& g, float hint, int* tw_out, std::vector<int32_t>* order_host,
-                 tw_stats* st) {
+                 tw_stats* st, int k_first) {
   const KeyClass kc = key_class_for(g.n);
   int rc = upload_graph(c, g, kc);
   if (rc) return rc;
   int32_t b[4];
   if ((rc = bounds_graph(c, g, b, true))) return rc;
-  const int lb = std::max(b[0], b[1]);
+  const int lb = std::max(std::max(b[0], b[1]), k_first);  // (every k below k_first answers no)
   int k0 = (int)std::lround(hint);
   k0 = std::min(std::max(k0, lb), g.n - 1);
   DecideResult R;

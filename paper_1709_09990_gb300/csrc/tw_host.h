@@ -193,9 +193,9 @@ int level_keys_graph(tw_ctx* c, const HostGraph& g, int k, int level, uint64_t* 
                      tw_stats* st);
 int bounds_graph(tw_ctx* c, const HostGraph& g, int32_t out[4], bool lower_only = false);
 int solve_graph(tw_ctx* c, const HostGraph& g, int* tw_out, int32_t* order, int32_t* td_parent, uint64_t* td_bags,
-                tw_stats* st, int k_first);
+                tw_stats* st, int k_first, bool try_fused = true);
 int solve_hinted(tw_ctx* c, const HostGraph& g, float hint, int* tw_out, std::vector<int32_t>* order_host,
-                 tw_stats* st);
+                 tw_stats* st, int k_first = 0);
 
 // ---- tw_batch_host.cu: many graphs
 int solve_batch_gpu(tw_ctx* c, const std::vector<HostGraph>& graphs, const std::vector<int>& idx,

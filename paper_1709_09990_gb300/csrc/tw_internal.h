@@ -216,7 +216,8 @@ struct BatchSolveArgs {
   unsigned long long* level_cnt;
   unsigned long long A, T;
   // results
-  int32_t* tw;                        // solve mode (-1 when the graph was left to the host)
+  int32_t* tw;                        // solve mode (-1 - the largest k known to answer no when
+                                      // the graph was left to the host)
   int32_t* orders;                    // solve mode, or null
   const int64_t* order_off;
   int32_t* status;                    // 0 done, 2 outgrew the workspace
