@@ -599,18 +599,25 @@ int run_batch_persistent(tw_ctx* c, const std::vector<HostGraph>& graphs, const 
     ooff[j] = order_off[q[j]];
     total_n = std::max<int64_t>(total_n, ooff[j] + hg.n);
   }
-  const int blocks = batch_solve_blocks(warps);
+  const int blocks = std::min(batch_solve_blocks(warps), G);
   // workspace: per block A keys and predecessor bytes, two tables of 2A slots
   const size_t room = c->mem_cap > total_bytes(c) ? c->mem_cap - total_bytes(c) : 0;
   const size_t budget = std::min<size_t>(room / 4, 32ull << 30);
-  // 2^16 states by default: a graph whose decide runs outgrow that is better
-  // served by the level-synchronous kernel, which spreads each level over the
-  // whole GPU, than by one block (measured on the batch workload's light
-  // graphs: 2^19 1.09 s, 2^17 0.67 s, 2^15 0.56 s, 2^13 0.54 s)
-  unsigned long long A = 1ull << 16;
+  // By default a run may hold 2^12 states: a graph whose decide runs outgrow
+  // that is better served by the level-synchronous kernel, which spreads each
+  // level over the whole GPU, than by one block (64 graphs of 12 to 24
+  // vertices: 10.8 ms with 2^16 states, 6.3 with 2^14, 5.6 with 2^12; 512 of 16
+  // to 48: 186, 173 and 170 ms).  Graphs of up to 16 vertices may hold 2^16:
+  // none of their runs outgrows that, so a batch of them is one launch.
+  constexpr int kOneLaunchN = 16;
+  bool one_launch = false;
+  for (int j = 0; j < G; ++j) one_launch = one_launch || ns[j] <= kOneLaunchN;
+  unsigned long long A = one_launch ? 1ull << 16 : 1ull << 12;
+  unsigned long long limit = 1ull << 12;  // for graphs above kOneLaunchN
   if (c->cfg.batch_arena_states > 0) {
     A = 1ull << 19;
     while (A > 4096 && A > (unsigned long long)c->cfg.batch_arena_states) A >>= 1;
+    limit = A;
   }
   while (A > 4096 && (size_t)blocks * (A * 41 + 4096) > budget) A >>= 1;
   const unsigned long long T = 2 * A;
@@ -651,6 +658,8 @@ int run_batch_persistent(tw_ctx* c, const std::vector<HostGraph>& graphs, const 
   a.max_probes = kBatchProbes;
   a.load_pct = 50;
   a.A = A;
+  a.limit = std::min(A, limit);
+  a.one_launch_n = kOneLaunchN;
   a.T = T;
   unsigned int* d_next = nullptr;
   unsigned long long* d_tot = nullptr;
@@ -789,7 +798,7 @@ int solve_batch_gpu(tw_ctx* c, const std::vector<HostGraph>& graphs, const std::
 }
 
 // Decide runs of many graphs at their own k: graphs with n <= 64 through the
-// batched kernel, the others (and any the batch evicts) one at a time through
+// batched kernels, the others (and any they evict) one at a time through
 // the single-graph path, with the Section 3.1 options and pruning turned off
 // so that every graph reports the plain method's level sets.
 int decide_batch_gpu(tw_ctx* c, const std::vector<HostGraph>& graphs, const std::vector<int>& idx,
@@ -820,10 +829,13 @@ int decide_batch_gpu(tw_ctx* c, const std::vector<HostGraph>& graphs, const std:
   dm.fp_xor = fp_xor;
   std::vector<int64_t> order_off(graphs.size(), 0);
   std::vector<int> htw(graphs.size(), -1);
-  int rc = c->cfg.batch_kernel == 1
-               ? run_batch(c, graphs, small, nullptr, order_off, htw.data(), nullptr, hst, st, &single, &dm)
-               : run_batch_persistent(c, graphs, small, nullptr, order_off, htw.data(), nullptr, hst, st, &single, &dm,
-                                      0);
+  std::vector<int> outgrown;
+  int rc = TW_OK;
+  if (c->cfg.batch_kernel == 1)
+    outgrown = small;
+  else
+    rc = run_batch_persistent(c, graphs, small, nullptr, order_off, htw.data(), nullptr, hst, st, &outgrown, &dm, 0);
+  if (rc == TW_OK) rc = run_batch(c, graphs, outgrown, nullptr, order_off, htw.data(), nullptr, hst, st, &single, &dm);
   if (rc) return rc;
   const tw_config saved = c->cfg;
   c->cfg.clique_skip = c->cfg.disjoint_paths = c->cfg.mmw_prune = 0;

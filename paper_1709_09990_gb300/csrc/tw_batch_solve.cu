@@ -99,13 +99,14 @@ __device__ __noinline__ bool block_decide(const BatchSolveArgs& a, const K* adj,
     *yes = true;
     return true;
   }
+  const unsigned long long most = n <= a.one_launch_n ? a.A : a.limit;
   unsigned long long off = 0, cnt = 1, prev_cnt = 0;
   for (int i = 0; i <= n - k - 2; ++i) {
     // the plan of the level in integer arithmetic (FP64 is slow on this part)
     unsigned long long table_est = 0, slots = 0;
     core::plan_level(cnt, prev_cnt, n, i, a.load_pct, &table_est, &slots);
     const unsigned long long out_off = off + cnt;
-    if (out_off >= a.A || a.A - out_off < table_est) return false;
+    if (out_off >= most || most - out_off < table_est) return false;
     if (slots > a.T) slots = a.T;
     const int t = i & 1;
     unsigned long long got = 0, gen = 0;
@@ -125,7 +126,7 @@ __device__ __noinline__ bool block_decide(const BatchSolveArgs& a, const K* adj,
       p.max_probes = a.max_probes;
       p.out_keys = w.arena + out_off;
       p.out_pred = w.pred + out_off;
-      p.out_cap = a.A - out_off;
+      p.out_cap = most - out_off;
       p.ctr = w.ctr;
       p.allowed = kones<K>();
       p.mmw = 0;

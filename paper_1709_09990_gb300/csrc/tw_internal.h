@@ -215,6 +215,8 @@ struct BatchSolveArgs {
   unsigned long long* level_off;
   unsigned long long* level_cnt;
   unsigned long long A, T;
+  unsigned long long limit;           // states a run may hold (A for graphs of up to one_launch_n
+  int one_launch_n;                   // vertices)
   // results
   int32_t* tw;                        // solve mode (-1 - the largest k known to answer no when
                                       // the graph was left to the host)
