@@ -215,8 +215,7 @@ int tw_features_batch(tw_ctx* c, const uint64_t* adj_concat, const int32_t* n, c
   int rc = load_batch(adj_concat, n, row_offset, num_graphs, &hn, &hoff, &hadj);
   if (rc) return rc;
   for (int g = 0; g < num_graphs; ++g) {
-    HostGraph tmp;
-    rc = validate(hadj.data() + hoff[g], hn[g], &tmp);
+    rc = validate_rows(hadj.data() + hoff[g], hn[g]);
     if (rc) return rc;
   }
   Stager S(c);

@@ -40,14 +40,28 @@ __device__ __forceinline__ void warp_argmin(int& val, int& idx) {
   }
 }
 
-__device__ __forceinline__ void load_rows(K128* rows, const unsigned long long* adj, int n, int W, int lane) {
+// Row u of a graph of W words a row.
+template <class K>
+__device__ __forceinline__ K load_row(const unsigned long long* adj, int u, int W);
+template <>
+__device__ __forceinline__ unsigned long long load_row<unsigned long long>(const unsigned long long* adj, int u, int) {
+  return adj[u];
+}
+template <>
+__device__ __forceinline__ K128 load_row<K128>(const unsigned long long* adj, int u, int W) {
+  return K128{adj[(size_t)u * W], W > 1 ? adj[(size_t)u * W + 1] : 0ull};
+}
+
+template <class K>
+__device__ __forceinline__ void load_rows(K* rows, const unsigned long long* adj, int n, int W, int lane) {
   for (int u = lane; u < n; u += 32)
-    rows[u] = K128{adj[(size_t)u * W], W > 1 ? adj[(size_t)u * W + 1] : 0ull};
+    rows[u] = load_row<K>(adj, u, W);
   __syncwarp();
 }
 
 // Minimum degree among alive vertices of `among` (lowest index on ties).
-__device__ __forceinline__ void min_degree(const K128* rows, K128 alive, K128 among, int n, int lane, int& d,
+template <class K>
+__device__ __forceinline__ void min_degree(const K* rows, K alive, K among, int n, int lane, int& d,
                                            int& v) {
   d = 1 << 30;
   v = -1;
@@ -62,58 +76,62 @@ __device__ __forceinline__ void min_degree(const K128* rows, K128 alive, K128 am
   warp_argmin(d, v);
 }
 
-__device__ int bound_mmd(K128* rows, const unsigned long long* adj, int n, int W, int lane) {
+template <class K>
+__device__ int bound_mmd(K* rows, const unsigned long long* adj, int n, int W, int lane) {
   load_rows(rows, adj, n, W, lane);
-  K128 alive = kfirst_n<K128>(n);
+  K alive = kfirst_n<K>(n);
   int lb = 0;
   for (int step = 0; step < n; ++step) {
     int d, v;
     min_degree(rows, alive, alive, n, lane, d, v);
     lb = max(lb, d);
-    alive &= ~kbit<K128>(v);
+    alive &= ~kbit<K>(v);
   }
   return lb;
 }
 
-__device__ int bound_mmd_plus(K128* rows, const unsigned long long* adj, int n, int W, int lane) {
+template <class K>
+__device__ int bound_mmd_plus(K* rows, const unsigned long long* adj, int n, int W, int lane) {
   load_rows(rows, adj, n, W, lane);
-  K128 alive = kfirst_n<K128>(n);
+  K alive = kfirst_n<K>(n);
   int lb = 0;
   while (kpopc(alive) >= 2) {
     int d, v;
     min_degree(rows, alive, alive, n, lane, d, v);
     lb = max(lb, d);
     if (d == 0) {
-      alive &= ~kbit<K128>(v);
+      alive &= ~kbit<K>(v);
       continue;
     }
-    const K128 nv = rows[v] & alive;
+    const K nv = rows[v] & alive;
     int du, u;
     min_degree(rows, alive, nv, n, lane, du, u);
     __syncwarp();
     for (int w = lane; w < n; w += 32) {
-      if (w == u) rows[w] |= nv & ~kbit<K128>(u);
-      else if (ktest(nv, w)) rows[w] |= kbit<K128>(u);
+      if (w == u) rows[w] |= nv & ~kbit<K>(u);
+      else if (ktest(nv, w)) rows[w] |= kbit<K>(u);
     }
     __syncwarp();
-    alive &= ~kbit<K128>(v);
+    alive &= ~kbit<K>(v);
   }
   return lb;
 }
 
 // Eliminates v: its alive neighbourhood becomes a clique.
-__device__ __forceinline__ void eliminate(K128* rows, K128& alive, int v, int n, int lane) {
-  const K128 nv = rows[v] & alive;
+template <class K>
+__device__ __forceinline__ void eliminate(K* rows, K& alive, int v, int n, int lane) {
+  const K nv = rows[v] & alive;
   __syncwarp();
   for (int w = lane; w < n; w += 32)
-    if (ktest(nv, w)) rows[w] |= nv & ~kbit<K128>(w);
+    if (ktest(nv, w)) rows[w] |= nv & ~kbit<K>(w);
   __syncwarp();
-  alive &= ~kbit<K128>(v);
+  alive &= ~kbit<K>(v);
 }
 
-__device__ int ub_min_degree(K128* rows, const unsigned long long* adj, int n, int W, int lane) {
+template <class K>
+__device__ int ub_min_degree(K* rows, const unsigned long long* adj, int n, int W, int lane) {
   load_rows(rows, adj, n, W, lane);
-  K128 alive = kfirst_n<K128>(n);
+  K alive = kfirst_n<K>(n);
   int width = 0;
   for (int step = 0; step < n; ++step) {
     int d, v;
@@ -124,21 +142,22 @@ __device__ int ub_min_degree(K128* rows, const unsigned long long* adj, int n, i
   return width;
 }
 
-__device__ int ub_min_fill(K128* rows, const unsigned long long* adj, int n, int W, int lane) {
+template <class K>
+__device__ int ub_min_fill(K* rows, const unsigned long long* adj, int n, int W, int lane) {
   load_rows(rows, adj, n, W, lane);
-  K128 alive = kfirst_n<K128>(n);
+  K alive = kfirst_n<K>(n);
   int width = 0;
   for (int step = 0; step < n; ++step) {
     int f = 1 << 30, v = -1;
     for (int u = lane; u < n; u += 32) {
       if (!ktest(alive, u)) continue;
-      const K128 nu = rows[u] & alive;
+      const K nu = rows[u] & alive;
       int missing2 = 0;
-      K128 t = nu;
+      K t = nu;
       while (!kempty(t)) {
         const int a = klowest(t);
         t = kdrop_lowest(t);
-        missing2 += kpopc(nu & ~rows[a] & ~kbit<K128>(a));
+        missing2 += kpopc(nu & ~rows[a] & ~kbit<K>(a));
       }
       const int fu = missing2 / 2;
       if (v < 0 || fu < f) {
@@ -153,18 +172,10 @@ __device__ int ub_min_fill(K128* rows, const unsigned long long* adj, int n, int
   return width;
 }
 
-__global__ void __launch_bounds__(kWarpsPerBlock * 32)
-    bounds_kernel(const unsigned long long* __restrict__ adj, const int32_t* __restrict__ ns,
-                  const int64_t* __restrict__ offs, int num_graphs, int32_t* out, float* feats, int lower_only) {
-  __shared__ K128 sRows[kWarpsPerBlock][128];
-  const int lane = threadIdx.x & 31;
-  const int warp = threadIdx.x >> 5;
-  const int g = blockIdx.x * kWarpsPerBlock + warp;
-  if (g >= num_graphs) return;
-  const int n = ns[g];
-  const int W = (n + 63) / 64;
-  const unsigned long long* a = adj + offs[g];
-  K128* rows = sRows[warp];
+// The bounds and features of graph g by one warp, on rows of type K.
+template <class K>
+__device__ __forceinline__ void graph_bounds(K* rows, const unsigned long long* a, int g, int n, int W, int lane,
+                                             int32_t* out, float* feats, int lower_only) {
   const int mmd = bound_mmd(rows, a, n, W, lane);
   const int mmdp = bound_mmd_plus(rows, a, n, W, lane);
   // (the greedy widths take most of the time; a k sweep needs only the lower bounds)
@@ -224,6 +235,26 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32)
       f[11] = (float)((double)(ubd + ubf) / (2.0 * dn));
     }
   }
+}
+
+// Graphs of up to 64 vertices work on 64-bit rows: half the instructions of a
+// step and half the shared-memory words.
+__global__ void __launch_bounds__(kWarpsPerBlock * 32)
+    bounds_kernel(const unsigned long long* __restrict__ adj, const int32_t* __restrict__ ns,
+                  const int64_t* __restrict__ offs, int num_graphs, int32_t* out, float* feats, int lower_only) {
+  __shared__ K128 sRows[kWarpsPerBlock][128];
+  const int lane = threadIdx.x & 31;
+  const int warp = threadIdx.x >> 5;
+  const int g = blockIdx.x * kWarpsPerBlock + warp;
+  if (g >= num_graphs) return;
+  const int n = ns[g];
+  const int W = (n + 63) / 64;
+  const unsigned long long* a = adj + offs[g];
+  if (n <= 64)
+    graph_bounds<unsigned long long>(reinterpret_cast<unsigned long long*>(sRows[warp]), a, g, n, W, lane, out, feats,
+                                     lower_only);
+  else
+    graph_bounds<K128>(sRows[warp], a, g, n, W, lane, out, feats, lower_only);
 }
 
 }  // namespace

@@ -159,19 +159,38 @@ int grow(tw_ctx* c, DevBuf* b, size_t need, size_t keep) {
   return TW_OK;
 }
 
-int validate(const uint64_t* rows, int n, HostGraph* g) {
+// Symmetric, no loops, no bit >= n: every edge rc with c > r must have its
+// mirror, and there must be as many bits below the diagonal as above it.
+int validate_rows(const uint64_t* rows, int n) {
   if (n < 1 || n > TW_MAX_N) return TW_ERR_INVALID;
   const int W = (n + 63) / 64;
-  g->n = n;
-  g->words = W;
-  g->rows.assign(rows, rows + (size_t)n * W);
+  long above = 0, below = 0;
   for (int r = 0; r < n; ++r)
-    for (int c = 0; c < W * 64; ++c) {
-      const bool bit = (g->rows[(size_t)r * W + (c >> 6)] >> (c & 63)) & 1ull;
-      if (!bit) continue;
-      if (c >= n || c == r) return TW_ERR_INVALID;
-      if (!((g->rows[(size_t)c * W + (r >> 6)] >> (r & 63)) & 1ull)) return TW_ERR_INVALID;
+    for (int w = 0; w < W; ++w) {
+      uint64_t x = rows[(size_t)r * W + w];
+      const int used = std::min(64, n - 64 * w);
+      if (used < 64 && (x >> used) != 0) return TW_ERR_INVALID;
+      // the bits of this word below the diagonal, then the diagonal
+      const int d = r - 64 * w;
+      const uint64_t low = d < 0 ? 0ull : (d >= 64 ? ~0ull : (1ull << d) - 1ull);
+      below += __builtin_popcountll(x & low);
+      x &= ~low;
+      if (d >= 0 && d < 64 && ((x >> d) & 1ull)) return TW_ERR_INVALID;
+      above += __builtin_popcountll(x);
+      for (; x; x &= x - 1) {
+        const int c = 64 * w + __builtin_ctzll(x);
+        if (!((rows[(size_t)c * W + (r >> 6)] >> (r & 63)) & 1ull)) return TW_ERR_INVALID;
+      }
     }
+  return above == below ? TW_OK : TW_ERR_INVALID;
+}
+
+int validate(const uint64_t* rows, int n, HostGraph* g) {
+  const int rc = validate_rows(rows, n);
+  if (rc) return rc;
+  g->n = n;
+  g->words = (n + 63) / 64;
+  g->rows.assign(rows, rows + (size_t)n * g->words);
   return TW_OK;
 }
 

@@ -180,6 +180,7 @@ int put_solution(tw_ctx* c, int n, int words, int32_t* order, int32_t* td_parent
 size_t total_bytes(const tw_ctx* c);
 int grow(tw_ctx* c, DevBuf* b, size_t need, size_t keep);
 int host_take(tw_ctx* c, size_t bytes, char** out);
+int validate_rows(const uint64_t* rows, int n);
 int validate(const uint64_t* rows, int n, HostGraph* g);
 int load_graph(const uint64_t* adj, int n, HostGraph* g);
 char* small_at(tw_ctx* c, size_t off);

@@ -32,6 +32,7 @@ available here; these seeded families stand in for them):
 from __future__ import annotations
 
 import math
+from array import array
 from typing import List, Sequence
 
 import numpy as np
@@ -316,13 +317,18 @@ def concat_rows_u64(graphs: Sequence[Sequence[int]]):
     Graph g's rows start at word ``row_offset[g]``; each of its n[g] rows has
     ceil(n[g]/64) words."""
     ns = np.array([len(g) for g in graphs], dtype=np.int32)
-    offs = np.zeros(len(graphs), dtype=np.int64)
-    total = 0
-    for g, adj in enumerate(graphs):
-        offs[g] = total
-        total += len(adj) * words_for(len(adj))
-    out = np.zeros(total, dtype=np.uint64)
-    for g, adj in enumerate(graphs):
-        w = words_for(len(adj))
-        out[offs[g]: offs[g] + len(adj) * w] = to_rows_u64(adj, w).reshape(-1)
-    return out, ns, offs
+    sizes = ns.astype(np.int64) * np.maximum(1, (ns + 63) // 64)
+    offs = np.cumsum(sizes) - sizes
+    out = array("Q")
+    for adj in graphs:
+        if len(adj) <= 64 and isinstance(adj, list):
+            # (one C call per graph; rows that are no 64-bit words go the general way)
+            try:
+                rows = array("Q", adj)
+            except (OverflowError, TypeError):
+                rows = None
+            if rows is not None:
+                out.extend(rows)
+                continue
+        out.frombytes(to_rows_u64(adj).tobytes())
+    return np.frombuffer(out, dtype=np.uint64) if len(out) else np.zeros(0, np.uint64), ns, offs
