@@ -128,16 +128,15 @@ typedef struct {
                              order, tw_decide_level and the decide runs of
                              tw_solve without outputs use it; a failed host
                              allocation is TW_ERR_CAPACITY.                      */
-  int fused_states;       /* tw_solve / tw_decide on graphs with n <= 64 first run
-                             the whole k sweep, walk and tree decomposition in one
-                             cooperative launch (barriers between levels; the
-                             decide runs k, k+1, k+2 of the sweep run at once in
-                             three groups of blocks, and the first of them that
-                             does not answer no decides, as in the sequential
-                             sweep) whose level arenas hold this many states; a run
+  int fused_states;       /* tw_solve / tw_decide first run the whole k sweep, walk
+                             and tree decomposition in one cooperative launch
+                             (barriers between levels; the decide runs k, k+1, k+2
+                             of the sweep run at once in three groups of blocks,
+                             and the first of them that does not answer no
+                             decides, as in the sequential sweep) whose level arenas hold this many states; a run
                              whose levels outgrow it goes on with the level loop
-                             from the k it reached.  0 = 2^20 states (the
-                             default), -1 = never.  Not used with clique_skip,
+                             from the k it reached.  0 = 2^20 states, 2^19 for
+                             n > 64 (the default), -1 = never.  Not used with clique_skip,
                              disjoint_paths, mmw_prune or spill_levels.  Results
                              are unchanged.                                      */
   int batch_kernel;       /* tw_solve_batch / tw_decide_batch: 0 = one persistent

@@ -126,6 +126,7 @@ __device__ __noinline__ bool block_decide(const BatchSolveArgs& a, const K* adj,
       p.max_probes = a.max_probes;
       p.out_keys = w.arena + out_off;
       p.out_pred = w.pred + out_off;
+      p.out_parent = nullptr;
       p.out_cap = most - out_off;
       p.ctr = w.ctr;
       p.allowed = kones<K>();

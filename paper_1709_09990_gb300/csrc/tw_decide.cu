@@ -1036,7 +1036,7 @@ unsigned long long graph_hash(const HostGraph& g) {
 }
 
 bool fused_eligible(const tw_ctx* c, const HostGraph& g) {
-  if (g.n > 64 || c->cfg.fused_states < 0 || c->cfg.clique_skip || c->cfg.disjoint_paths || c->cfg.mmw_prune ||
+  if (c->cfg.fused_states < 0 || c->cfg.clique_skip || c->cfg.disjoint_paths || c->cfg.mmw_prune ||
       c->cfg.spill_levels)
     return false;
   const unsigned long long h = graph_hash(g);
@@ -1061,16 +1061,22 @@ int run_fused(tw_ctx* c, const HostGraph& g, KeyClass kc, int k0, int k_last, De
   constexpr int kGroups = 3;
   static_assert(kGroups <= kFusedMaxGroups, "the fused launch holds at most kFusedMaxGroups groups");
   const int G = std::max(1, std::min(kGroups, k_last - k0 + 1));
+  // (128-bit states: half the states, the same bytes)
   const unsigned long long A =
-      c->cfg.fused_states > 0 ? (unsigned long long)c->cfg.fused_states : (1ull << 20);
+      c->cfg.fused_states > 0 ? (unsigned long long)c->cfg.fused_states : (kc == kKey128 ? 1ull << 19 : 1ull << 20);
   const unsigned long long T = 2 * A + 1024;
   const size_t st_bytes = (sizeof(FusedState) + 255) & ~size_t(255);
-  const size_t tb = ((size_t)T * 8 + 255) & ~size_t(255);  // sized for 64-bit states
-  const size_t kb = ((size_t)A * 8 + 255) & ~size_t(255);
-  const size_t pb = ((size_t)A + 255) & ~size_t(255);
+  const size_t unit = kc == kKey128 ? 16 : 8;  // bytes per slot and key (32-bit states: room for 64)
+  const size_t tb = ((size_t)T * unit + 255) & ~size_t(255);
+  const size_t kb = ((size_t)A * unit + 255) & ~size_t(255);
+  const size_t pb = ((size_t)A * 4 + 255) & ~size_t(255);
   const size_t group_bytes = st_bytes + 2 * tb + kb + pb;
   const size_t need = (size_t)kGroups * group_bytes;
   *status = 0;
+  if (c->fused_unit != (int)unit) {
+    c->fused_clean = false;  // the groups' tables lie elsewhere
+    c->fused_unit = (int)unit;
+  }
   if (c->fused.bytes < need) {
     c->fused_clean = false;
     int rc = grow(c, &c->fused, need, 0);
@@ -1105,7 +1111,7 @@ int run_fused(tw_ctx* c, const HostGraph& g, KeyClass kc, int k0, int k_last, De
     f.table0[j] = gbase + st_bytes;
     f.table1[j] = gbase + st_bytes + tb;
     f.keys[j] = gbase + st_bytes + 2 * tb;
-    f.pred[j] = reinterpret_cast<uint8_t*>(gbase + st_bytes + 2 * tb + kb);
+    f.parent_of[j] = reinterpret_cast<uint32_t*>(gbase + st_bytes + 2 * tb + kb);
   }
   f.arena_cap = A;
   f.table_cap = T;
@@ -1120,6 +1126,7 @@ int run_fused(tw_ctx* c, const HostGraph& g, KeyClass kc, int k0, int k_last, De
   }
   f.tables_clean = 1;
   for (int j = 0; j < G; ++j) TW_CK(cudaMemsetAsync(f.st[j], 0, sizeof(FusedState), c->stream));
+  TW_CK(cudaMemsetAsync(&f.st[0]->settled_k, 0x7f, sizeof(int), c->stream));
   const bool timed = c->cfg.time_kernels != 0;
   if (timed) TW_CK(cudaEventRecord(c->ev0, c->stream));
   TW_LAUNCH(c, launch_fused_solve(f, c->stream));

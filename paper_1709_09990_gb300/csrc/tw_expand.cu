@@ -26,6 +26,8 @@
 // longest probe sequence and to the counter.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "tw_expand_core.cuh"
 #include "tw_internal.h"
 #include "tw_keys.cuh"
@@ -110,6 +112,7 @@ cudaError_t launch_expand_t(const ExpandLaunch& a, cudaStream_t s) {
   p.max_probes = a.max_probes;
   p.out_keys = static_cast<K*>(a.out_keys);
   p.out_pred = a.out_pred;
+  p.out_parent = nullptr;
   p.out_cap = a.out_cap;
   p.ctr = a.ctr;
   p.allowed = core::kfrom_words<K>(a.allowed[0], a.allowed[1]);
@@ -118,7 +121,9 @@ cudaError_t launch_expand_t(const ExpandLaunch& a, cudaStream_t s) {
   p.range = a.range;
   if (a.n_in == 0) return cudaSuccess;
   const unsigned long long chunks = (a.n_in + 31ull) / 32ull;
-  const unsigned long long blocks_needed = (chunks + kWarps - 1) / kWarps;
+  // (small levels are dealt out in chunks of fewer than 32 states)
+  const unsigned long long spread = std::min<unsigned long long>(a.n_in, core::kSpreadWarps);
+  const unsigned long long blocks_needed = (std::max(chunks, spread) + kWarps - 1) / kWarps;
   if (a.ranges > 0) {
     const unsigned long long need4 = (chunks + 3) / 4;
     return launch_ranged<K>(p, static_cast<K*>(a.out_tail), a.out_split, need4, s);

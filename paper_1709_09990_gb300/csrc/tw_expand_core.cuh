@@ -550,7 +550,8 @@ struct ExpandParams {
   unsigned long long table_slots;
   int max_probes;
   K* out_keys;
-  uint8_t* out_pred;
+  uint8_t* out_pred;        // predecessor vertex of each new set, or (kParent)
+  uint32_t* out_parent;     // the index of its parent in the input level
   unsigned long long out_cap;
   LevelCounters* ctr;
   K allowed;  // vertices that may be added (all by default)
@@ -617,8 +618,13 @@ __device__ __forceinline__ void add_warp_count(unsigned long long count, const i
 // With kGroup the level is expanded by a group of the grid's blocks (block
 // group_block of group_blocks) instead of the whole grid.  Ranged kernels may
 // continue the output list in out_tail from position out_split on.
-template <class K, int kWarps, bool kMMW = false, bool kRanged = false,
-          bool kBlockLocal = false, bool kKeysL2 = false, bool kGroup = false>
+//
+// A level of fewer than 32 states per warp is dealt out in smaller chunks, to at
+// most kSpreadWarps warps (each adds to the level's counter once): a chunk takes
+// as long as its rounds of 32 pairs, one after the other.
+constexpr unsigned kSpreadWarps = 1024;
+template <class K, int kWarps, bool kMMW = false, bool kRanged = false, bool kBlockLocal = false,
+          bool kKeysL2 = false, bool kGroup = false, bool kParent = false>
 __device__ __forceinline__ void expand_level(const ExpandParams<K>& p, K* sAdj, WarpScratch<K>* scratch,
                                              const unsigned group_block = 0, const unsigned group_blocks = 0,
                                              K* out_tail = nullptr, const unsigned long long out_split = 0) {
@@ -630,35 +636,38 @@ __device__ __forceinline__ void expand_level(const ExpandParams<K>& p, K* sAdj, 
   const K valid = kfirst_n<K>(p.n);
   unsigned long long generated = 0;
   int staged = 0;
-  const unsigned long long n_chunks = (p.n_in + 31ull) / 32ull;
   const unsigned long long blk = kGroup ? (unsigned long long)group_block : (unsigned long long)blockIdx.x;
   const unsigned long long nblk = kGroup ? (unsigned long long)group_blocks : (unsigned long long)gridDim.x;
   const unsigned long long first = kBlockLocal ? (unsigned long long)warp : blk * kWarps + warp;
   const unsigned long long stride = kBlockLocal ? (unsigned long long)kWarps : nblk * kWarps;
-  LevelOut<K, false> out;
+  const unsigned spread = (unsigned)min(stride, (unsigned long long)kSpreadWarps);
+  const unsigned per = p.n_in < 32ull * spread ? max(1u, ((unsigned)p.n_in + spread - 1u) / spread) : 32u;
+  const unsigned long long n_chunks = per == 32u ? (p.n_in + 31ull) / 32ull : ((unsigned)p.n_in + per - 1u) / per;
+  LevelOut<K, kParent> out;
   out.keys = p.out_keys;
   out.pred = p.out_pred;
-  out.parent = nullptr;
+  out.parent = p.out_parent;
   out.parent_base = 0;
   out.cap = p.out_cap;
   out.count = &p.ctr->out_count;
   out.overflow = &p.ctr->overflow;
   for (unsigned long long chunk = first; chunk < n_chunks; chunk += stride) {
-    const unsigned long long idx = chunk * 32ull + lane;
-    const bool active = idx < p.n_in;
+    const unsigned long long idx = chunk * per + lane;
+    const bool active = (unsigned)lane < per && idx < p.n_in;
+    if (kParent) out.parent_base = (uint32_t)(chunk * per);
     const K S = active ? (kKeysL2 ? kload_cg(&p.in_keys[idx]) : kload_cs(&p.in_keys[idx])) : valid;
     // (minor-min-width pruning drops some parents, so it extends by every
     // feasible vertex)
     Candidates<K> c = start_chunk<K, !kMMW, kMMW>(S, active, sAdj, valid, p.allowed, p.n, p.k, lane, w);
     do {
       const int total = build_queue<K>(c, lane, w);
-      generated += (unsigned long long)search_insert<K, false, kRanged>(w, total, staged, lane, sAdj, p.k, p.table,
+      generated += (unsigned long long)search_insert<K, kParent, kRanged>(w, total, staged, lane, sAdj, p.k, p.table,
                                                                            p.table_slots, p.max_probes, out, p.ranges,
                                                                            p.range, out_tail, out_split);
       __syncwarp();
     } while (__any_sync(kFull, any_left(c)));
   }
-  flush_stage<K, false, kRanged>(w, staged, lane, out, out_tail, out_split);
+  flush_stage<K, kParent, kRanged>(w, staged, lane, out, out_tail, out_split);
   add_warp_count(generated, lane, &p.ctr->generated);
 }
 
@@ -713,6 +722,26 @@ __device__ __forceinline__ void walk_block(const K* __restrict__ keys, const uin
       if (!ktest(fin, v)) order[pos++] = v;
   }
   __syncthreads();
+}
+
+// The backward walk by one thread through parent indices: the added vertex is
+// the bit in which a set and its parent differ.  Two dependent loads per level
+// (scanning a level of 10^5 sets for the predecessor took a block 50 us).
+template <class K>
+__device__ __forceinline__ void walk_parents(const K* __restrict__ keys, const uint32_t* __restrict__ parent,
+                                             const unsigned long long* level_off, int last, int n, int32_t* order) {
+  unsigned long long idx = 0;
+  K S = kload_cg(&keys[__ldcg(&level_off[last])]);
+  const K fin = S;
+  for (int j = last; j >= 1; --j) {
+    idx = __ldcg(&parent[__ldcg(&level_off[j]) + idx]);
+    const K prev = kload_cg(&keys[__ldcg(&level_off[j - 1]) + idx]);
+    order[j - 1] = kindex(S ^ prev);
+    S = prev;
+  }
+  int pos = last;
+  for (int v = 0; v < n; ++v)
+    if (!ktest(fin, v)) order[pos++] = v;
 }
 
 // Tree decomposition from an ordering, by one block (thread per vertex):

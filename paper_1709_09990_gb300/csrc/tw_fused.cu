@@ -8,7 +8,8 @@
 // 32 states plus a barrier.  Here the grid is split into groups of blocks and
 // consecutive decide runs of the sweep (k, k+1, ...) run at the same time,
 // one per group, so the sweep takes about as many level steps as its longest
-// run instead of their sum.  Within a group every block runs the same loop:
+// run instead of their sum; a run stops as soon as a smaller k has answered yes
+// (the runs above tw are the large ones: on G(44, 0.5) they took 16 of 21 ms).  Within a group every block runs the same loop:
 // expand level i (the group's blocks take the chunks of 32 states in turn,
 // the kernel body of tw_expand_core.cuh) while emptying the table the
 // previous level used, then one barrier of the group.  Every block reads the
@@ -101,7 +102,7 @@ struct FusedArgs {
   int n, words64, k0, k_last, max_probes, load_pct, groups, tables_clean;
   const int32_t* lb_dev;              // or null: lower bounds on the device that raise k0
   K* keys[kFusedMaxGroups];           // per group: level arena
-  uint8_t* pred[kFusedMaxGroups];
+  uint32_t* parent_of[kFusedMaxGroups];  // index of each set's parent in its level
   unsigned long long arena_cap;
   K* table[kFusedMaxGroups][2];
   unsigned long long table_cap;       // slots of each table
@@ -113,8 +114,9 @@ struct FusedArgs {
 
 // One decide run at bound k by the blocks of one group (gb = this block's
 // index in the group, nb = the group's blocks).  Returns 0 (no), 1 (yes),
-// 2 (gave up: a level would not fit the arena or a table) or -2 (a barrier
-// gave up); *last = index of the final level built.
+// 2 (gave up: a level would not fit the arena or a table), -1 (stopped: a
+// smaller k has answered yes or given up) or -2 (a barrier gave up); *last =
+// index of the final level built.
 template <class K>
 __device__ int group_decide(const FusedArgs<K>& a, int grp, unsigned int gb, unsigned int nb, int k,
                             unsigned long long dirty[2], int* last, K* sAdj, core::WarpScratch<K>* sScratch) {
@@ -162,7 +164,8 @@ __device__ int group_decide(const FusedArgs<K>& a, int grp, unsigned int gb, uns
     p.table = a.table[grp][t];
     p.max_probes = a.max_probes;
     p.out_keys = keys + out_off;
-    p.out_pred = a.pred[grp] + out_off;
+    p.out_pred = nullptr;
+    p.out_parent = a.parent_of[grp] + out_off;
     p.out_cap = a.arena_cap - out_off;
     p.ctr = &st->ctr[i + 1];
     p.allowed = kones<K>();
@@ -172,14 +175,19 @@ __device__ int group_decide(const FusedArgs<K>& a, int grp, unsigned int gb, uns
     unsigned long long got = 0;
     for (int attempt = 0;; ++attempt) {
       p.table_slots = slots;
-      core::expand_level<K, kFusedWarps, false, false, false, true, true>(p, sAdj, sScratch, gb, nb);
+      core::expand_level<K, kFusedWarps, false, false, false, true, true, true>(p, sAdj, sScratch, gb, nb);
       // meanwhile empty the table the previous level used
       for (unsigned long long j = gtid; j < dirty[1 - t]; j += gthreads) a.table[grp][1 - t][j] = kones<K>();
       dirty[1 - t] = 0;
       dirty[t] = slots;
+      // a run above a k that has answered (or given up) is not needed: one
+      // thread looks and tells the group at the barrier
+      if (gb == 0 && threadIdx.x == 0)
+        st->ctr[i + 1].pad[0] = k > *(volatile int*)&a.st[0]->settled_k ? 1u : 0u;
       if (!barrier_wait(&st->arrive, &st->gen, nb, error)) return -2;
       got = __ldcg(&st->ctr[i + 1].out_count);
       const unsigned int ovf = __ldcg(&st->ctr[i + 1].overflow);
+      if (__ldcg(&st->ctr[i + 1].pad[0]) != 0u) return -1;
       if (ovf == 0u) break;  // every pair placed, every new set appended: the level is exact
       // the arena is full, or the largest table is: the host goes on
       if ((ovf & 1u) || got > p.out_cap || slots >= a.table_cap || attempt > 0) return 2;
@@ -224,8 +232,6 @@ __global__ void __launch_bounds__(kFusedWarps * 32, ResidentWarps<K>::value / kF
   __shared__ core::WarpScratch<K> sScratch[kFusedWarps];
   __shared__ K128 sTdAdj[128];
   __shared__ int sPos[128];
-  __shared__ K sWalk;
-  __shared__ int sFound;
   FusedState* st0 = a.st[0];
   const unsigned int nb = gridDim.x / (unsigned int)a.groups;
   const int grp = (int)(blockIdx.x / nb);  // == groups for the idle remainder
@@ -248,6 +254,7 @@ __global__ void __launch_bounds__(kFusedWarps * 32, ResidentWarps<K>::value / kF
       if (gb == 0 && threadIdx.x == 0) {
         a.st[grp]->result = result;
         a.st[grp]->run_last = last;
+        if (result == 1 || result == 2) atomicMin(&st0->settled_k, k);
       }
     }
     if (!barrier_wait(&st0->w_arrive, &st0->w_gen, gridDim.x, &st0->error)) return;
@@ -317,9 +324,9 @@ __global__ void __launch_bounds__(kFusedWarps * 32, ResidentWarps<K>::value / kF
   // the backward walk through the answering group's levels, then the tree
   // decomposition
   FusedState* sg = a.st[answer_grp];
-  core::walk_block<K>(a.keys[answer_grp], a.pred[answer_grp], sg->level_off, sg->level_cnt, answer_last, a.n,
-                      a.order, &sWalk, &sFound);
-  __threadfence_block();
+  if (threadIdx.x == 0)
+    core::walk_parents<K>(a.keys[answer_grp], a.parent_of[answer_grp], sg->level_off, answer_last, a.n, a.order);
+  __syncthreads();
   core::td_block(a.adj64, a.n, a.words64, a.order, a.parent, a.bags, sTdAdj, sPos);
   if (threadIdx.x == 0) {
     st0->status = 1;
@@ -346,7 +353,7 @@ cudaError_t launch_t(const FusedLaunch& f, cudaStream_t s) {
   for (int g = 0; g < kFusedMaxGroups; ++g) {
     const int h = g < a.groups ? g : 0;
     a.keys[g] = static_cast<K*>(f.keys[h]);
-    a.pred[g] = f.pred[h];
+    a.parent_of[g] = f.parent_of[h];
     a.table[g][0] = static_cast<K*>(f.table0[h]);
     a.table[g][1] = static_cast<K*>(f.table1[h]);
     a.st[g] = f.st[h];
@@ -379,7 +386,7 @@ cudaError_t launch_fused_solve(const FusedLaunch& f, cudaStream_t s) {
   switch (f.kc) {
     case kKey32: return launch_t<uint32_t>(f, s);
     case kKey64: return launch_t<unsigned long long>(f, s);
-    default: return cudaErrorInvalidValue;
+    default: return launch_t<K128>(f, s);
   }
 }
 

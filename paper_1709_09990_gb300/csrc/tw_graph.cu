@@ -126,6 +126,7 @@ cudaError_t expand_t(const GraphState* st, const ExpandLaunch& a, cudaStream_t s
   p.max_probes = a.max_probes;
   p.out_keys = static_cast<K*>(a.out_keys);
   p.out_pred = a.out_pred;
+  p.out_parent = nullptr;
   p.out_cap = 0;
   p.ctr = a.ctr;
   p.allowed = core::kfrom_words<K>(a.allowed[0], a.allowed[1]);

@@ -99,6 +99,7 @@ struct tw_ctx {
   // fused small solves: state, two tables and the level arena in one buffer,
   // a pinned mirror of the state, and the graphs whose fused run gave up
   DevBuf fused;
+  int fused_unit = 0;        // bytes per slot of its layout (8, or 16 for 128-bit states)
   bool fused_clean = false;  // every table slot of the fused buffer is empty
   FusedState* h_fused = nullptr;
   unsigned char* h_out = nullptr;  // pinned mirror of the small buffer's order .. bags region

@@ -152,7 +152,7 @@ cudaError_t launch_graph_expand(const GraphState* st, const ExpandLaunch& base, 
 constexpr int kFusedMaxGroups = 4;  // decide runs of the sweep in flight at once
 
 // Device state of one group of a fused solve (zeroed by the host before the
-// launch).  Group 0's state also holds the solve's summary and the window
+// launch, but for settled_k).  Group 0's state also holds the solve's summary and the window
 // barrier of the whole grid.
 struct FusedState {
   unsigned long long level_off[130];  // arena index of level j of the group's run
@@ -169,10 +169,12 @@ struct FusedState {
                                       // index of the final level of the deciding run and
                                       // the group that ran it
   int k_start;                        // group 0: the first k of the sweep
+  int settled_k;                      // group 0: the smallest k that answered yes or gave up
+                                      // (set to INT_MAX by the launch)
 };
 
 struct FusedLaunch {
-  KeyClass kc;                        // kKey32 or kKey64
+  KeyClass kc;
   const void* adj;                    // n rows in the state layout
   const unsigned long long* adj64;    // n rows of words64 words
   int n, words64, k0, k_last, max_probes, load_pct;  // decide runs at k0 .. k_last
@@ -181,7 +183,7 @@ struct FusedLaunch {
   const int32_t* lb_dev;              // or null: the sweep starts at max(k0, lb_dev[0], lb_dev[1])
                                       // (lower bounds written by a kernel earlier on the stream)
   void* keys[kFusedMaxGroups];        // per group: arena of arena_cap states
-  uint8_t* pred[kFusedMaxGroups];
+  uint32_t* parent_of[kFusedMaxGroups];
   unsigned long long arena_cap;
   void* table0[kFusedMaxGroups];      // per group: two tables of table_cap slots
   void* table1[kFusedMaxGroups];
@@ -193,7 +195,7 @@ struct FusedLaunch {
 };
 
 // The k sweep from k0, the walk and the tree decomposition of one graph
-// (n <= 64) in one cooperative launch; see tw_fused.cu.
+// in one cooperative launch; see tw_fused.cu.
 cudaError_t launch_fused_solve(const FusedLaunch& f, cudaStream_t s);
 
 // ---- persistent batched solve (tw_batch_solve.cu) ----------------------------

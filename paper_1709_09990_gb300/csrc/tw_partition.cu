@@ -321,6 +321,7 @@ cudaError_t emit_t(const ExpandLaunch& a, const PartitionBufs& pb, cudaStream_t 
   p.max_probes = a.max_probes;
   p.out_keys = static_cast<K*>(a.out_keys);
   p.out_pred = a.out_pred;
+  p.out_parent = nullptr;
   p.out_cap = a.out_cap;
   p.ctr = a.ctr;
   p.allowed = core::kfrom_words<K>(a.allowed[0], a.allowed[1]);
