@@ -78,7 +78,8 @@ __device__ void block_fingerprint(const K* keys, unsigned long long count, unsig
 // With fp_sum / fp_xor (decide mode) the level fingerprints are written.
 template <int kWarps>
 __device__ __noinline__ bool block_decide(const BatchSolveArgs& a, const K* adj, int n, int k, Work& w, K* sAdj,
-                             core::WarpScratch<K>* sScratch, unsigned long long* sRed, bool* yes, int* last,
+                             core::WarpScratch<K>* sScratch, const unsigned long long* sSets,
+                             unsigned long long* sRed, bool* yes, int* last,
                              unsigned long long* stats, unsigned long long* fp_sum, unsigned long long* fp_xor) {
   for (int t = 0; t < 2; ++t) {
     for (unsigned long long j = threadIdx.x; j < w.dirty[t]; j += blockDim.x) w.table[t][j] = kones<K>();
@@ -104,7 +105,7 @@ __device__ __noinline__ bool block_decide(const BatchSolveArgs& a, const K* adj,
   for (int i = 0; i <= n - k - 2; ++i) {
     // the plan of the level in integer arithmetic (FP64 is slow on this part)
     unsigned long long table_est = 0, slots = 0;
-    core::plan_level(cnt, prev_cnt, n, i, a.load_pct, &table_est, &slots);
+    core::plan_level(cnt, prev_cnt, n, i, a.load_pct, sSets[i + 1], &table_est, &slots);
     const unsigned long long out_off = off + cnt;
     if (out_off >= most || most - out_off < table_est) return false;
     if (slots > a.T) slots = a.T;
@@ -178,6 +179,7 @@ __global__ void __launch_bounds__(kWarps * 32, 24 / kWarps) batch_solve_kernel(c
   __shared__ K sAdj[64];
   __shared__ core::WarpScratch<K> sScratch[kWarps];
   __shared__ unsigned long long sRed[2 * kWarps];
+  __shared__ unsigned long long sSets[65];  // C(n, j), capped
   __shared__ K sWalk;
   __shared__ int sFound;
   __shared__ int sGraph;
@@ -201,12 +203,13 @@ __global__ void __launch_bounds__(kWarps * 32, 24 / kWarps) batch_solve_kernel(c
     if (g >= a.num_graphs) break;
     const int n = a.n[g];
     const K* adj = a.adj + (size_t)g * 64;
+    for (int j = threadIdx.x; j <= n; j += blockDim.x) sSets[j] = core::binom_capped(n, j, core::kSetsCap);
     bool yes = false;
     int last = 0;
     if (a.decide_mode) {
       unsigned long long* fs = a.fp_sum ? a.fp_sum + (size_t)g * 129 : nullptr;
       unsigned long long* fx = a.fp_xor ? a.fp_xor + (size_t)g * 129 : nullptr;
-      const bool ok = block_decide<kWarps>(a, adj, n, a.k_start[g], w, sAdj, sScratch, sRed, &yes, &last,
+      const bool ok = block_decide<kWarps>(a, adj, n, a.k_start[g], w, sAdj, sScratch, sSets, sRed, &yes, &last,
                                            stats, fs, fx);
       ++runs;
       if (threadIdx.x == 0) {
@@ -225,7 +228,7 @@ __global__ void __launch_bounds__(kWarps * 32, 24 / kWarps) batch_solve_kernel(c
     int yes_min = INT_MAX, no_max = lb - 1, yes_in_arena = -1;
     bool ok = true;
     for (;;) {
-      ok = block_decide<kWarps>(a, adj, n, k, w, sAdj, sScratch, sRed, &yes, &last, stats, nullptr, nullptr);
+      ok = block_decide<kWarps>(a, adj, n, k, w, sAdj, sScratch, sSets, sRed, &yes, &last, stats, nullptr, nullptr);
       ++runs;
       if (!ok) break;
       if (yes) {
@@ -240,7 +243,7 @@ __global__ void __launch_bounds__(kWarps * 32, 24 / kWarps) batch_solve_kernel(c
     }
     if (ok && yes_in_arena != yes_min) {
       // the last run was a no: run the yes at tw again for its levels
-      ok = block_decide<kWarps>(a, adj, n, yes_min, w, sAdj, sScratch, sRed, &yes, &last, stats, nullptr,
+      ok = block_decide<kWarps>(a, adj, n, yes_min, w, sAdj, sScratch, sSets, sRed, &yes, &last, stats, nullptr,
                                 nullptr);
       ++runs;
     }

@@ -762,7 +762,7 @@ int run_decide_graph(tw_ctx* c, KeyClass kc, int n, int k, DecideResult* R, bool
     ++nodes;
     if (err == cudaSuccess)
       err = launch_graph_plan(c->d_gstate, c->d_ctr, arena_cap, table_cap, partition_threshold_bytes(c), n, k,
-                              load_pct, w, 1, c->stream);
+                              load_pct, w, 0, c->stream);
     ++nodes;
     for (int i = 0; i <= n - k - 2 && err == cudaSuccess; ++i) {
       err = launch_graph_clear(kc, c->d_gstate, c->table.ptr, c->stream);
@@ -772,7 +772,7 @@ int run_decide_graph(tw_ctx* c, KeyClass kc, int n, int k, DecideResult* R, bool
         err = cudaEventRecordWithFlags(ev[2 * i + 1], c->stream, cudaEventRecordExternal);
       if (err == cudaSuccess)
         err = launch_graph_plan(c->d_gstate, c->d_ctr, arena_cap, table_cap, partition_threshold_bytes(c), n, k,
-                                load_pct, w, 0, c->stream);
+                                load_pct, w, i + 1, c->stream);
       nodes += 3;
     }
     const cudaError_t end = cudaStreamEndCapture(c->stream, &graph);

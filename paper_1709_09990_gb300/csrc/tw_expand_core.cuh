@@ -359,20 +359,14 @@ struct LevelOut {
   unsigned int* overflow;  // bit 0: output full, bit 1: probe limit
 };
 
-// Moves the warp's staged new sets to the output list: one atomic add for all of
-// them.  (Every add of a level goes to the same counter, which takes about one
-// in 2.6 ns; with one add per 64 pairs that was the whole time of a level, with
-// one per 200 new sets it no longer shows.)  With kRanged no predecessor is
-// stored and output positions from split on go to tail[position - split] when
-// tail is given (a list continued in a second buffer).
+// Writes the warp's staged new sets to the output list from position b on.  With
+// kRanged no predecessor is stored and output positions from split on go to
+// tail[position - split] when tail is given (a list continued in a second
+// buffer).
 template <class K, bool kParent, bool kRanged>
-__device__ __forceinline__ void flush_stage(WarpScratch<K>& w, int& staged, const int lane,
-                                            const LevelOut<K, kParent>& out, K* tail, const unsigned long long split) {
-  if (staged == 0) return;
-  __syncwarp();
-  unsigned long long b = 0;
-  if (lane == 0) b = atomicAdd(out.count, (unsigned long long)staged);
-  b = __shfl_sync(kFull, b, 0);
+__device__ __forceinline__ void store_stage(const WarpScratch<K>& w, const int staged, const unsigned long long b,
+                                            const int lane, const LevelOut<K, kParent>& out, K* tail,
+                                            const unsigned long long split) {
   for (int j = lane; j < staged; j += 32) {
     const unsigned long long o = b + (unsigned long long)j;
     if (o < out.cap) {
@@ -388,6 +382,21 @@ __device__ __forceinline__ void flush_stage(WarpScratch<K>& w, int& staged, cons
       atomicOr(out.overflow, 1u);
     }
   }
+}
+
+// Moves the warp's staged new sets to the output list: one atomic add for all of
+// them.  (Every add of a level goes to the same counter, which takes about one
+// in 2.6 ns; with one add per 64 pairs that was the whole time of a level, with
+// one per 200 new sets it no longer shows.)
+template <class K, bool kParent, bool kRanged>
+__device__ __forceinline__ void flush_stage(WarpScratch<K>& w, int& staged, const int lane,
+                                            const LevelOut<K, kParent>& out, K* tail, const unsigned long long split) {
+  if (staged == 0) return;
+  __syncwarp();
+  unsigned long long b = 0;
+  if (lane == 0) b = atomicAdd(out.count, (unsigned long long)staged);
+  b = __shfl_sync(kFull, b, 0);
+  store_stage<K, kParent, kRanged>(w, staged, b, lane, out, tail, split);
   staged = 0;
   __syncwarp();
 }
@@ -563,7 +572,7 @@ struct ExpandParams {
 // C(n, r), or cap when it is at least cap.  The products run over
 // min(r, n - r) steps, along which b = C(n - r + j, j) only grows and each
 // division is exact, so with cap <= 2^40 nothing overflows.
-__device__ __forceinline__ unsigned long long binom_capped(int n, int r, unsigned long long cap) {
+__host__ __device__ __forceinline__ unsigned long long binom_capped(int n, int r, unsigned long long cap) {
   if (r < 0 || r > n) return 0ull;
   if (r > n - r) r = n - r;
   unsigned long long b = 1ull;
@@ -579,15 +588,21 @@ __device__ __forceinline__ unsigned long long binom_capped(int n, int r, unsigne
 // ratio cnt / prev_cnt clamped to [1/4, n - i] (n at i = 0), plus 25% and
 // 1024, at most the number of sets level i+1 can have; slots = that at
 // load_pct percent, at least 64.  The ratio is exact integer arithmetic below
-// 2^32 sets and single precision above.
+// 2^32 sets and single precision above.  sets_max = C(n, i+1), capped at
+// kSetsCap (64-bit divisions take a thread 0.1 us each: the callers compute the
+// binomials once per run or graph, not level by level, which took 1 to 3 us).
+constexpr unsigned long long kSetsCap = 1ull << 40;
 __device__ __forceinline__ void plan_level(unsigned long long cnt, unsigned long long prev_cnt, int n, int i,
-                                           int load_pct, unsigned long long* table_est, unsigned long long* slots) {
+                                           int load_pct, unsigned long long sets_max, unsigned long long* table_est,
+                                           unsigned long long* slots) {
   const unsigned long long most = cnt * (unsigned long long)(n - i);
-  const unsigned long long bound = min(most, binom_capped(n, i + 1, 1ull << 40)) + 1ull;
+  const unsigned long long bound = min(most, sets_max) + 1ull;
   unsigned long long est = (unsigned long long)n;
   if (i > 0) {
     if (prev_cnt == 0)
       est = cnt;
+    else if (cnt < (1ull << 16) && prev_cnt < (1ull << 32))
+      est = ((unsigned)cnt * (unsigned)cnt) / (unsigned)prev_cnt;
     else if (cnt < (1ull << 32))
       est = cnt * cnt / prev_cnt;
     else
@@ -596,7 +611,9 @@ __device__ __forceinline__ void plan_level(unsigned long long cnt, unsigned long
     est = min(est, most);
   }
   *table_est = min(est + est / 4ull + 1024ull, bound);
-  *slots = max(64ull, (*table_est * 100ull + (unsigned long long)load_pct - 1ull) / (unsigned long long)load_pct);
+  *slots = max(64ull, load_pct == 50 ? 2ull * *table_est
+                                     : (*table_est * 100ull + (unsigned long long)load_pct - 1ull) /
+                                           (unsigned long long)load_pct);
 }
 
 // Adds the lanes' counts and, in lane 0, adds the sum to *total.
@@ -616,7 +633,8 @@ __device__ __forceinline__ void add_warp_count(unsigned long long count, const i
 // With kKeysL2 the input keys are read through L2 only: persistent kernels,
 // whose arena other SMs rewrite while stale lines may sit in this SM's L1.
 // With kGroup the level is expanded by a group of the grid's blocks (block
-// group_block of group_blocks) instead of the whole grid.  Ranged kernels may
+// group_block of group_blocks) instead of the whole grid, and the caller has
+// put the adjacency rows in sAdj.  Ranged kernels may
 // continue the output list in out_tail from position out_split on.
 //
 // A level of fewer than 32 states per warp is dealt out in smaller chunks, to at
@@ -628,8 +646,10 @@ template <class K, int kWarps, bool kMMW = false, bool kRanged = false, bool kBl
 __device__ __forceinline__ void expand_level(const ExpandParams<K>& p, K* sAdj, WarpScratch<K>* scratch,
                                              const unsigned group_block = 0, const unsigned group_blocks = 0,
                                              K* out_tail = nullptr, const unsigned long long out_split = 0) {
-  for (int i = threadIdx.x; i < p.n; i += blockDim.x) sAdj[i] = p.adj[i];
-  __syncthreads();
+  if (!kGroup) {
+    for (int i = threadIdx.x; i < p.n; i += blockDim.x) sAdj[i] = p.adj[i];
+    __syncthreads();
+  }
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
   WarpScratch<K>& w = scratch[warp];
@@ -666,6 +686,35 @@ __device__ __forceinline__ void expand_level(const ExpandParams<K>& p, K* sAdj, 
                                                                            p.range, out_tail, out_split);
       __syncwarp();
     } while (__any_sync(kFull, any_left(c)));
+  }
+  if (kGroup) {
+    // the block's last sets and its pair count with one atomic add each: at a
+    // small level the adds to the two counters, 2.6 ns each, are on the way to
+    // the group's barrier
+    __shared__ int sStaged[kWarps];
+    __shared__ unsigned int sPairs[kWarps];
+    __shared__ unsigned long long sFirst;
+    const unsigned int pairs = __reduce_add_sync(kFull, (unsigned)generated);  // (a lane's pairs of a level: 32 bits)
+    if (lane == 0) {
+      sStaged[warp] = staged;
+      sPairs[warp] = pairs;
+    }
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      unsigned int sets = 0;
+      unsigned long long all = 0;
+      for (int x = 0; x < kWarps; ++x) {
+        sets += (unsigned)sStaged[x];
+        all += sPairs[x];
+      }
+      if (all) atomicAdd(&p.ctr->generated, all);
+      sFirst = sets ? atomicAdd(out.count, (unsigned long long)sets) : 0ull;
+    }
+    __syncthreads();
+    unsigned long long b = sFirst;
+    for (int x = 0; x < warp; ++x) b += (unsigned long long)sStaged[x];
+    store_stage<K, kParent, kRanged>(w, staged, b, lane, out, out_tail, out_split);
+    return;
   }
   flush_stage<K, kParent, kRanged>(w, staged, lane, out, out_tail, out_split);
   add_warp_count(generated, lane, &p.ctr->generated);

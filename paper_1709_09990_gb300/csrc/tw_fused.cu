@@ -24,8 +24,9 @@
 // own loop from that k.  Every barrier wait is bounded: a barrier that does
 // not complete within a second (the global timer) sets an error flag, and all
 // blocks return.
-#include <cooperative_groups.h>
 #include <cuda_runtime.h>
+
+#include <algorithm>
 
 #include "tw_expand_core.cuh"
 #include "tw_internal.h"
@@ -35,8 +36,11 @@ namespace tw {
 namespace {
 
 using core::ExpandParams;
-using core::ResidentWarps;
-constexpr int kFusedWarps = 4;
+// Warps per block: 8, two blocks per SM (800 warps and a hundred arrivals per
+// group of a third of the grid); 4 for 128-bit sets, whose scratch of 8 warps
+// would not fit the static shared memory.
+template <class K>
+constexpr int kFusedWarps = KeyTraits<K>::kBits <= 64 ? 8 : 4;
 constexpr unsigned long long kBarrierNs = 1000000000ull;  // a barrier wait gives up after a second
 
 __device__ __forceinline__ unsigned long long global_ns() {
@@ -55,44 +59,34 @@ __device__ __forceinline__ unsigned int atom_add_acq_rel(unsigned int* p, unsign
   asm volatile("atom.acq_rel.gpu.global.add.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
   return old;
 }
-__device__ __forceinline__ void red_add_release(unsigned int* p, unsigned int v) {
-  asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
-__device__ __forceinline__ void st_relaxed(unsigned int* p, unsigned int v) {
-  asm volatile("st.relaxed.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
-
-// Bounded barrier over `count` co-resident blocks of a cooperative launch,
-// on the counter `arrive` and the generation word `gen`.  The block's threads
-// meet at a block barrier; its thread 0 arrives with an acquire-release add
-// (which also publishes the block's writes); the last block to arrive resets
-// the count and advances the generation with a release; the others poll the
-// generation with acquire loads, or give up after kBarrierNs and set *error.
-// Returns false once any block has given up.
-__device__ bool barrier_wait(unsigned int* arrive, unsigned int* gen, unsigned int count, unsigned int* error) {
+// Bounded barrier over `count` co-resident blocks of a cooperative launch, on a
+// counter that only grows.  The block's threads meet at a block barrier; its
+// thread 0 arrives with an acquire-release add (which also publishes the
+// block's writes) and polls the counter with acquire loads until the round's
+// last arrival, or gives up after kBarrierNs: it sets *error and the counter's
+// top bit, which every block of this barrier sees.  `round` counts this block's
+// barriers on the counter.  Returns false once a block has given up.
+constexpr unsigned int kGaveUp = 0x80000000u;
+__device__ bool barrier_wait(unsigned int* arrive, unsigned int& round, unsigned int count, unsigned int* error,
+                             unsigned int* sSeen) {
   __syncthreads();
+  const unsigned int target = ++round * count;
   if (threadIdx.x == 0) {
-    const unsigned int g = ld_acquire(gen);
-    const unsigned int prev = atom_add_acq_rel(arrive, 1u);
-    if (prev == count - 1) {
-      st_relaxed(arrive, 0u);
-      red_add_release(gen, 1u);
-    } else {
-      const unsigned long long t0 = global_ns();
-      unsigned int polls = 0;
-      while (ld_acquire(gen) == g) {
-        if ((++polls & 255u) == 0u) {
-          if (ld_acquire(error) != 0u) break;
-          if (global_ns() - t0 > kBarrierNs) {
-            atomicExch(error, 1u);
-            break;
-          }
-        }
+    unsigned int seen = atom_add_acq_rel(arrive, 1u) + 1u;
+    const unsigned long long t0 = global_ns();
+    unsigned int polls = 0;
+    while (!(seen & kGaveUp) && seen < target) {
+      seen = ld_acquire(arrive);
+      if ((++polls & 255u) == 0u && (ld_acquire(error) != 0u || global_ns() - t0 > kBarrierNs)) {
+        atomicExch(error, 1u);
+        atomicOr(arrive, kGaveUp);
+        seen |= kGaveUp;
       }
     }
+    *sSeen = seen;
   }
   __syncthreads();
-  return *(volatile unsigned int*)error == 0u;
+  return !(*sSeen & kGaveUp);
 }
 
 template <class K>
@@ -119,7 +113,8 @@ struct FusedArgs {
 // index of the final level built.
 template <class K>
 __device__ int group_decide(const FusedArgs<K>& a, int grp, unsigned int gb, unsigned int nb, int k,
-                            unsigned long long dirty[2], int* last, K* sAdj, core::WarpScratch<K>* sScratch) {
+                            unsigned long long dirty[2], int* last, K* sAdj, core::WarpScratch<K>* sScratch,
+                            const unsigned long long* sSets, unsigned int& round, unsigned int* sSeen) {
   FusedState* st = a.st[grp];
   unsigned int* error = &a.st[0]->error;
   K* keys = a.keys[grp];
@@ -142,7 +137,7 @@ __device__ int group_decide(const FusedArgs<K>& a, int grp, unsigned int gb, uns
       st->run_states = st->run_candidates = st->run_generated = 0ull;
     }
   }
-  if (!barrier_wait(&st->arrive, &st->gen, nb, error)) return -2;
+  if (!barrier_wait(&st->arrive, round, nb, error, sSeen)) return -2;
   *last = 0;
   if (k >= n - 1) return 1;
   unsigned long long off = 0, cnt = 1, prev_cnt = 0;
@@ -151,7 +146,7 @@ __device__ int group_decide(const FusedArgs<K>& a, int grp, unsigned int gb, uns
     // (integer arithmetic: this part's FP64 rate is a small fraction of its
     // integer rate)
     unsigned long long table_est = 0, slots = 0;
-    core::plan_level(cnt, prev_cnt, n, i, a.load_pct, &table_est, &slots);
+    core::plan_level(cnt, prev_cnt, n, i, a.load_pct, sSets[i + 1], &table_est, &slots);
     const unsigned long long out_off = off + cnt;
     if (slots > a.table_cap || out_off >= a.arena_cap || a.arena_cap - out_off < table_est) return 2;
     const int t = i & 1;
@@ -175,7 +170,8 @@ __device__ int group_decide(const FusedArgs<K>& a, int grp, unsigned int gb, uns
     unsigned long long got = 0;
     for (int attempt = 0;; ++attempt) {
       p.table_slots = slots;
-      core::expand_level<K, kFusedWarps, false, false, false, true, true, true>(p, sAdj, sScratch, gb, nb);
+      core::expand_level<K, kFusedWarps<K>, false, false, false, true, true, true>(p, sAdj, sScratch, gb,
+                                                                                                nb);
       // meanwhile empty the table the previous level used
       for (unsigned long long j = gtid; j < dirty[1 - t]; j += gthreads) a.table[grp][1 - t][j] = kones<K>();
       dirty[1 - t] = 0;
@@ -184,7 +180,7 @@ __device__ int group_decide(const FusedArgs<K>& a, int grp, unsigned int gb, uns
       // thread looks and tells the group at the barrier
       if (gb == 0 && threadIdx.x == 0)
         st->ctr[i + 1].pad[0] = k > *(volatile int*)&a.st[0]->settled_k ? 1u : 0u;
-      if (!barrier_wait(&st->arrive, &st->gen, nb, error)) return -2;
+      if (!barrier_wait(&st->arrive, round, nb, error, sSeen)) return -2;
       got = __ldcg(&st->ctr[i + 1].out_count);
       const unsigned int ovf = __ldcg(&st->ctr[i + 1].overflow);
       if (__ldcg(&st->ctr[i + 1].pad[0]) != 0u) return -1;
@@ -193,11 +189,11 @@ __device__ int group_decide(const FusedArgs<K>& a, int grp, unsigned int gb, uns
       if ((ovf & 1u) || got > p.out_cap || slots >= a.table_cap || attempt > 0) return 2;
       // a pair reached the probe limit: run the level again with the largest
       // table, once every block has read the counters
-      if (!barrier_wait(&st->arrive, &st->gen, nb, error)) return -2;
+      if (!barrier_wait(&st->arrive, round, nb, error, sSeen)) return -2;
       for (unsigned long long j = gtid; j < slots; j += gthreads) a.table[grp][t][j] = kones<K>();
       if (gb == 0 && threadIdx.x == 0) st->ctr[i + 1] = LevelCounters{};
       slots = a.table_cap;
-      if (!barrier_wait(&st->arrive, &st->gen, nb, error)) return -2;
+      if (!barrier_wait(&st->arrive, round, nb, error, sSeen)) return -2;
     }
     if (gb == 0 && threadIdx.x == 0) {
       st->level_off[i + 1] = out_off;
@@ -226,12 +222,18 @@ __device__ int group_decide(const FusedArgs<K>& a, int grp, unsigned int gb, uns
 // starts.  The first block of the group that answered walks back and builds
 // the tree decomposition.
 template <class K>
-__global__ void __launch_bounds__(kFusedWarps * 32, ResidentWarps<K>::value / kFusedWarps)
+__global__ void __launch_bounds__(kFusedWarps<K> * 32, 16 / kFusedWarps<K>)
     fused_solve_kernel(const FusedArgs<K> a) {
   __shared__ K sAdj[KeyTraits<K>::kBits];
-  __shared__ core::WarpScratch<K> sScratch[kFusedWarps];
+  __shared__ core::WarpScratch<K> sScratch[kFusedWarps<K>];
+  __shared__ unsigned long long sSets[129];  // C(n, j), capped
+  __shared__ unsigned int sSeen;
   __shared__ K128 sTdAdj[128];
   __shared__ int sPos[128];
+  for (int i = threadIdx.x; i < a.n; i += blockDim.x) sAdj[i] = a.adj[i];
+  for (int j = threadIdx.x; j <= a.n; j += blockDim.x) sSets[j] = core::binom_capped(a.n, j, core::kSetsCap);
+  __syncthreads();
+  unsigned int round = 0, w_round = 0;  // this block's barriers on its group's and the grid's counter
   FusedState* st0 = a.st[0];
   const unsigned int nb = gridDim.x / (unsigned int)a.groups;
   const int grp = (int)(blockIdx.x / nb);  // == groups for the idle remainder
@@ -248,7 +250,7 @@ __global__ void __launch_bounds__(kFusedWarps * 32, ResidentWarps<K>::value / kF
       const int k = k_base + grp;
       int result = -1, last = 0;
       if (k <= a.k_last) {
-        result = group_decide<K>(a, grp, gb, nb, k, dirty, &last, sAdj, sScratch);
+        result = group_decide<K>(a, grp, gb, nb, k, dirty, &last, sAdj, sScratch, sSets, round, &sSeen);
         if (result == -2) return;
       }
       if (gb == 0 && threadIdx.x == 0) {
@@ -257,7 +259,7 @@ __global__ void __launch_bounds__(kFusedWarps * 32, ResidentWarps<K>::value / kF
         if (result == 1 || result == 2) atomicMin(&st0->settled_k, k);
       }
     }
-    if (!barrier_wait(&st0->w_arrive, &st0->w_gen, gridDim.x, &st0->error)) return;
+    if (!barrier_wait(&st0->w_arrive, w_round, gridDim.x, &st0->error, &sSeen)) return;
     // the same decision in every block
     int counted = 0;
     for (int g = 0; g < a.groups && status == 0; ++g) {
@@ -291,7 +293,7 @@ __global__ void __launch_bounds__(kFusedWarps * 32, ResidentWarps<K>::value / kF
       }
     }
     // the results are read by every block before the next window overwrites them
-    if (status == 0 && !barrier_wait(&st0->w_arrive, &st0->w_gen, gridDim.x, &st0->error)) return;
+    if (status == 0 && !barrier_wait(&st0->w_arrive, w_round, gridDim.x, &st0->error, &sSeen)) return;
   }
   // leave the group's tables empty for the next launch
   if (grp < a.groups) {
@@ -368,16 +370,14 @@ cudaError_t launch_t(const FusedLaunch& f, cudaStream_t s) {
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
   if (!coop) return cudaErrorNotSupported;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fused_solve_kernel<K>, kFusedWarps * 32, 0);
+  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fused_solve_kernel<K>, kFusedWarps<K> * 32, 0);
   if (per_sm < 1) return cudaErrorNotSupported;
-  // two blocks per SM: each of the three groups has about a hundred blocks
-  // (400 warps, so a level of a few thousand states is one chunk per warp)
-  // and a barrier of a group takes about a hundred arrivals
-  const int grid = sms * (per_sm >= 2 ? 2 : 1);
+  // 16 warps per SM
+  const int grid = sms * std::min(per_sm, 16 / kFusedWarps<K>);
   if (grid < a.groups) return cudaErrorNotSupported;
   void* args[] = {&a};
   return cudaLaunchCooperativeKernel(reinterpret_cast<void*>(fused_solve_kernel<K>), dim3(grid),
-                                     dim3(kFusedWarps * 32), args, 0, s);
+                                     dim3(kFusedWarps<K> * 32), args, 0, s);
 }
 
 }  // namespace

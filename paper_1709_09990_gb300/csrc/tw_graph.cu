@@ -33,7 +33,7 @@ __global__ void graph_init_kernel(GraphState* st, K* keys) {
 // loop; the output may use the rest of the arena.
 __global__ void graph_plan_kernel(GraphState* st, LevelCounters* ctr, unsigned long long arena_cap,
                                   unsigned long long table_cap, unsigned long long direct_table_bytes, int n, int k,
-                                  int load_pct, int w, int first) {
+                                  int load_pct, int w, int first, unsigned long long sets_max) {
   if (st->done || st->bail) return;
   if (!first) {
     const unsigned long long cnt = ctr->out_count;
@@ -64,7 +64,8 @@ __global__ void graph_plan_kernel(GraphState* st, LevelCounters* ctr, unsigned l
   // (integer plan: a chain of FP64 divisions in one thread costs about ten
   // microseconds per level on this part)
   unsigned long long table_est = 0, slots = 0;
-  core::plan_level(st->level_cnt[i], i > 0 ? st->level_cnt[i - 1] : 0ull, n, i, load_pct, &table_est, &slots);
+  core::plan_level(st->level_cnt[i], i > 0 ? st->level_cnt[i - 1] : 0ull, n, i, load_pct, sets_max,
+                   &table_est, &slots);
   const unsigned long long out_off = st->level_off[i] + st->level_cnt[i];
   // levels for the partitioned insert, and levels that do not fit, go back
   // to the host loop
@@ -157,9 +158,9 @@ cudaError_t launch_graph_init(KeyClass kc, GraphState* st, void* keys, cudaStrea
 
 cudaError_t launch_graph_plan(GraphState* st, LevelCounters* ctr, unsigned long long arena_cap,
                               unsigned long long table_cap, unsigned long long direct_table_bytes, int n, int k,
-                              int load_pct, int key_bytes, int first, cudaStream_t s) {
+                              int load_pct, int key_bytes, int level, cudaStream_t s) {
   graph_plan_kernel<<<1, 1, 0, s>>>(st, ctr, arena_cap, table_cap, direct_table_bytes, n, k, load_pct, key_bytes,
-                                    first);
+                                    level == 0 ? 1 : 0, core::binom_capped(n, level + 1, core::kSetsCap));
   return cudaGetLastError();
 }
 

@@ -140,9 +140,11 @@ struct GraphState {
 };
 
 cudaError_t launch_graph_init(KeyClass kc, GraphState* st, void* keys, cudaStream_t s);
+// Plans level -> level + 1 of the run (unless it has ended); level > 0 first
+// records the level just built.
 cudaError_t launch_graph_plan(GraphState* st, LevelCounters* ctr, unsigned long long arena_cap,
                               unsigned long long table_cap, unsigned long long direct_table_bytes, int n, int k,
-                              int load_pct, int key_bytes, int first, cudaStream_t s);
+                              int load_pct, int key_bytes, int level, cudaStream_t s);
 cudaError_t launch_graph_clear(KeyClass kc, const GraphState* st, void* table, cudaStream_t s);
 // base: in_keys/out_keys = the arena, out_pred = the predecessor arena; the
 // level fields come from st.
@@ -160,8 +162,8 @@ struct FusedState {
   LevelCounters ctr[130];             // counters of the expansion that built level j
   unsigned long long states_expanded, candidates, generated;  // group 0: over the counted runs
   unsigned long long run_states, run_candidates, run_generated;  // the group's current run
-  unsigned int arrive, gen, error;    // the group's barrier; error (group 0): a wait gave up
-  unsigned int w_arrive, w_gen;       // group 0: barrier of all blocks at the end of a window
+  unsigned int arrive, error;         // the group's barrier; error (group 0): a wait gave up
+  unsigned int w_arrive;              // group 0: barrier of all blocks at the end of a window
   int result, run_last;               // the group's run: 0 no, 1 yes, 2 gave up, -1 not run;
                                       // index of its final level
   int status;                         // group 0: 1 finished, 2 gave up at k = last
