@@ -141,6 +141,8 @@ void tw_destroy(tw_ctx* c) {
   if (c->d_gstate) cudaFree(c->d_gstate);
   if (c->h_gstate) cudaFreeHost(c->h_gstate);
   if (c->h_out) cudaFreeHost(c->h_out);
+  if (c->h_up) cudaFreeHost(c->h_up);
+  if (c->ev_up) cudaEventDestroy(c->ev_up);
   if (c->ev0) cudaEventDestroy(c->ev0);
   if (c->ev1) cudaEventDestroy(c->ev1);
   if (c->own_stream && c->stream) cudaStreamDestroy(c->stream);

@@ -257,7 +257,33 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32)
     graph_bounds<K128>(sRows[warp], a, g, n, W, lane, out, feats, lower_only);
 }
 
+// The two lower bounds of one graph of n vertices, a warp each: both are chains
+// of warp argmins, and a solve waits for them.
+__global__ void __launch_bounds__(64) lower_bounds_kernel(const unsigned long long* __restrict__ adj, int n,
+                                                          int32_t* out) {
+  __shared__ K128 sRows[2][128];
+  const int lane = threadIdx.x & 31;
+  const int warp = threadIdx.x >> 5;
+  const int W = (n + 63) / 64;
+  int lb;
+  if (n <= 64) {
+    unsigned long long* rows = reinterpret_cast<unsigned long long*>(sRows[warp]);
+    lb = warp == 0 ? bound_mmd(rows, adj, n, W, lane) : bound_mmd_plus(rows, adj, n, W, lane);
+  } else {
+    lb = warp == 0 ? bound_mmd(sRows[warp], adj, n, W, lane) : bound_mmd_plus(sRows[warp], adj, n, W, lane);
+  }
+  if (lane == 0) {
+    out[warp] = lb;
+    out[2 + warp] = -1;
+  }
+}
+
 }  // namespace
+
+cudaError_t launch_lower_bounds(const unsigned long long* adj, int n, int32_t* out, cudaStream_t s) {
+  lower_bounds_kernel<<<1, 64, 0, s>>>(adj, n, out);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_bounds(const unsigned long long* adj, const int32_t* n, const int64_t* row_offset, int num_graphs,
                           int32_t* out, float* feats, cudaStream_t s, int lower_only) {

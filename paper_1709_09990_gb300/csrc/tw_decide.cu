@@ -1051,9 +1051,10 @@ bool fused_eligible(const tw_ctx* c, const HostGraph& g) {
 // buffer); 2 = gave up at k = *bail_k (the runs before it answered no), and
 // the graph is remembered so that later solves skip the fused attempt; 0 =
 // not run (its buffers do not fit the memory cap).
-// Totals of every run go into st.
+// Totals of every run go into st.  With want_out the ordering and decomposition
+// are copied to the pinned mirror h_out along with the state.
 int run_fused(tw_ctx* c, const HostGraph& g, KeyClass kc, int k0, int k_last, DecideResult* R, int* status,
-              int* answer_k, int* bail_k, tw_stats* st, const int32_t* lb_dev) {
+              int* answer_k, int* bail_k, tw_stats* st, const int32_t* lb_dev, bool want_out) {
   NvtxRange range("tw fused solve n=%d k0=%d", g.n, k0);
   const size_t w = key_bytes(kc);
   // decide runs in flight at once: k0, k0+1, k0+2 (the sweep from a lower
@@ -1070,8 +1071,9 @@ int run_fused(tw_ctx* c, const HostGraph& g, KeyClass kc, int k0, int k_last, De
   const size_t tb = ((size_t)T * unit + 255) & ~size_t(255);
   const size_t kb = ((size_t)A * unit + 255) & ~size_t(255);
   const size_t pb = ((size_t)A * 4 + 255) & ~size_t(255);
-  const size_t group_bytes = st_bytes + 2 * tb + kb + pb;
-  const size_t need = (size_t)kGroups * group_bytes;
+  // the groups' states side by side, then each group's tables, keys and parents
+  const size_t group_bytes = 2 * tb + kb + pb;
+  const size_t need = (size_t)kGroups * (st_bytes + group_bytes);
   *status = 0;
   if (c->fused_unit != (int)unit) {
     c->fused_clean = false;  // the groups' tables lie elsewhere
@@ -1084,7 +1086,7 @@ int run_fused(tw_ctx* c, const HostGraph& g, KeyClass kc, int k0, int k_last, De
     if (rc) return rc;
   }
   if (!c->h_fused) {
-    if (cudaHostAlloc(reinterpret_cast<void**>(&c->h_fused), kFusedMaxGroups * sizeof(FusedState),
+    if (cudaHostAlloc(reinterpret_cast<void**>(&c->h_fused), (size_t)kGroups * st_bytes,
                       cudaHostAllocDefault) != cudaSuccess) {
       c->h_fused = nullptr;
       cudaGetLastError();
@@ -1106,12 +1108,13 @@ int run_fused(tw_ctx* c, const HostGraph& g, KeyClass kc, int k0, int k_last, De
   f.groups = G;
   f.lb_dev = lb_dev;
   for (int j = 0; j < kFusedMaxGroups; ++j) {
-    char* gbase = base + (size_t)std::min(j, kGroups - 1) * group_bytes;
-    f.st[j] = reinterpret_cast<FusedState*>(gbase);
-    f.table0[j] = gbase + st_bytes;
-    f.table1[j] = gbase + st_bytes + tb;
-    f.keys[j] = gbase + st_bytes + 2 * tb;
-    f.parent_of[j] = reinterpret_cast<uint32_t*>(gbase + st_bytes + 2 * tb + kb);
+    const size_t at = (size_t)std::min(j, kGroups - 1);
+    char* gbase = base + kGroups * st_bytes + at * group_bytes;
+    f.st[j] = reinterpret_cast<FusedState*>(base + at * st_bytes);
+    f.table0[j] = gbase;
+    f.table1[j] = gbase + tb;
+    f.keys[j] = gbase + 2 * tb;
+    f.parent_of[j] = reinterpret_cast<uint32_t*>(gbase + 2 * tb + kb);
   }
   f.arena_cap = A;
   f.table_cap = T;
@@ -1125,15 +1128,19 @@ int run_fused(tw_ctx* c, const HostGraph& g, KeyClass kc, int k0, int k_last, De
     c->fused_clean = true;
   }
   f.tables_clean = 1;
-  for (int j = 0; j < G; ++j) TW_CK(cudaMemsetAsync(f.st[j], 0, sizeof(FusedState), c->stream));
-  TW_CK(cudaMemsetAsync(&f.st[0]->settled_k, 0x7f, sizeof(int), c->stream));
+  TW_CK(cudaMemsetAsync(base, 0, G * st_bytes, c->stream));
   const bool timed = c->cfg.time_kernels != 0;
   if (timed) TW_CK(cudaEventRecord(c->ev0, c->stream));
   TW_LAUNCH(c, launch_fused_solve(f, c->stream));
   if (timed) TW_CK(cudaEventRecord(c->ev1, c->stream));
-  TW_CK(cudaMemcpyAsync(c->h_fused, f.st[0], sizeof(FusedState), cudaMemcpyDeviceToHost, c->stream));
+  TW_CK(cudaMemcpyAsync(c->h_fused, base, G * st_bytes, cudaMemcpyDeviceToHost, c->stream));
+  if (want_out) {
+    const int rc = fetch_solution(c);
+    if (rc) return rc;
+  }
   TW_CK(cudaStreamSynchronize(c->stream));
   const FusedState& h = *c->h_fused;
+  c->h_out_fresh = want_out && h.error == 0u && h.status == 1 && h.tw >= 0;
   c->fused_clean = h.error == 0u;  // a launch that ran to its end empties the tables it used
   if (h.error) return TW_ERR_TIMEOUT;  // a barrier wait gave up
   *status = h.status;
@@ -1152,12 +1159,8 @@ int run_fused(tw_ctx* c, const HostGraph& g, KeyClass kc, int k0, int k_last, De
   }
   // the levels of the deciding run are in its group's state and arena
   const int grp = std::min(std::max(h.group, 0), G - 1);
-  const FusedState* hl = &h;
-  if (grp != 0) {
-    TW_CK(cudaMemcpyAsync(c->h_fused + 1, f.st[grp], sizeof(FusedState), cudaMemcpyDeviceToHost, c->stream));
-    TW_CK(cudaStreamSynchronize(c->stream));
-    hl = c->h_fused + 1;
-  }
+  const FusedState* hl =
+      reinterpret_cast<const FusedState*>(reinterpret_cast<const char*>(c->h_fused) + (size_t)grp * st_bytes);
   *answer_k = h.tw;
   const int last_k = h.tw >= 0 ? h.tw : k_last;
   R->levels.clear();
@@ -1258,11 +1261,11 @@ int decide_graph(tw_ctx* c, const HostGraph& g, int k, int* yes, int32_t* order,
     int status = 0, ans = -1, bail_k = -1;
     tw_stats tmp;
     std::memset(&tmp, 0, sizeof(tmp));
-    rc = run_fused(c, g, kc, k, k, &R, &status, &ans, &bail_k, &tmp, nullptr);
+    rc = run_fused(c, g, kc, k, k, &R, &status, &ans, &bail_k, &tmp, nullptr, order != nullptr);
     if (rc) return rc;
     if (status == 1) {
       if (R.yes && order) {
-        rc = put_from_device(c, order, small_at(c, SmallLayout().order), (size_t)g.n * 4);
+        rc = put_solution(c, g.n, g.words, order, nullptr, nullptr);
         if (rc) return rc;
       }
       TW_CK(cudaStreamSynchronize(c->stream));
@@ -1365,9 +1368,29 @@ int level_keys_graph(tw_ctx* c, const HostGraph& g, int k, int level, uint64_t* 
   return TW_OK;
 }
 
+// Launches the lower bounds (MMD, MMD+) of the uploaded graph into the small
+// buffer's bounds slot without waiting for them; returns their device
+// address.
+int start_lower_bounds(tw_ctx* c, const HostGraph& g, const int32_t** d_bounds) {
+  SmallLayout L;
+  int32_t* d_out = reinterpret_cast<int32_t*>(small_at(c, L.bounds));
+  TW_LAUNCH(c, launch_lower_bounds(reinterpret_cast<const unsigned long long*>(small_at(c, L.adj64)), g.n, d_out,
+                                   c->stream));
+  *d_bounds = d_out;
+  return TW_OK;
+}
+
 int bounds_graph(tw_ctx* c, const HostGraph& g, int32_t out[4], bool lower_only) {
   SmallLayout L;
   int32_t* d_out = reinterpret_cast<int32_t*>(small_at(c, L.bounds));
+  if (lower_only) {
+    const int32_t* unused = nullptr;
+    const int rc = start_lower_bounds(c, g, &unused);
+    if (rc) return rc;
+    TW_CK(cudaMemcpyAsync(out, d_out, 16, cudaMemcpyDeviceToHost, c->stream));
+    TW_CK(cudaStreamSynchronize(c->stream));
+    return TW_OK;
+  }
   int32_t* d_n = d_out + 4;
   int64_t* d_off = reinterpret_cast<int64_t*>(small_at(c, L.bounds + 64));
   const int32_t nn = g.n;
@@ -1375,28 +1398,9 @@ int bounds_graph(tw_ctx* c, const HostGraph& g, int32_t out[4], bool lower_only)
   TW_CK(cudaMemcpyAsync(d_n, &nn, 4, cudaMemcpyHostToDevice, c->stream));
   TW_CK(cudaMemcpyAsync(d_off, &off, 8, cudaMemcpyHostToDevice, c->stream));
   TW_LAUNCH(c, launch_bounds(reinterpret_cast<const unsigned long long*>(small_at(c, L.adj64)), d_n, d_off, 1, d_out,
-                      nullptr, c->stream, lower_only ? 1 : 0));
+                      nullptr, c->stream));
   TW_CK(cudaMemcpyAsync(out, d_out, 16, cudaMemcpyDeviceToHost, c->stream));
   TW_CK(cudaStreamSynchronize(c->stream));
-  return TW_OK;
-}
-
-// Launches the lower bounds (MMD, MMD+) of the uploaded graph into the small
-// buffer's bounds slot without waiting for them; returns their device
-// address.
-int launch_lower_bounds(tw_ctx* c, const HostGraph& g, const int32_t** d_bounds) {
-  SmallLayout L;
-  int32_t* d_out = reinterpret_cast<int32_t*>(small_at(c, L.bounds));
-  int32_t* d_n = d_out + 4;
-  int64_t* d_off = reinterpret_cast<int64_t*>(small_at(c, L.bounds + 64));
-  // (n and the row offset go through the context's pinned counter block)
-  c->h_ctr->out_count = (unsigned long long)(unsigned)g.n;
-  c->h_ctr->generated = 0ull;
-  TW_CK(cudaMemcpyAsync(d_n, &c->h_ctr->out_count, 4, cudaMemcpyHostToDevice, c->stream));
-  TW_CK(cudaMemcpyAsync(d_off, &c->h_ctr->generated, 8, cudaMemcpyHostToDevice, c->stream));
-  TW_LAUNCH(c, launch_bounds(reinterpret_cast<const unsigned long long*>(small_at(c, L.adj64)), d_n, d_off, 1, d_out,
-                             nullptr, c->stream, 1));
-  *d_bounds = d_out;
   return TW_OK;
 }
 
@@ -1425,9 +1429,9 @@ int solve_graph(tw_ctx* c, const HostGraph& g, int* tw_out, int32_t* order, int3
     // the fused solve reads the lower bounds on the device: no host round
     // trip between the bounds and the sweep
     const int32_t* d_bounds = nullptr;
-    if ((rc = launch_lower_bounds(c, g, &d_bounds))) return rc;
+    if ((rc = start_lower_bounds(c, g, &d_bounds))) return rc;
     int status = 0, ans = -1, bail_k = -1;
-    rc = run_fused(c, g, kc, k_first, g.n - 1, &R, &status, &ans, &bail_k, st, d_bounds);
+    rc = run_fused(c, g, kc, k_first, g.n - 1, &R, &status, &ans, &bail_k, st, d_bounds, want_walk);
     if (rc) return rc;
     if (status == 1) {
       tw = ans;
@@ -1449,7 +1453,7 @@ int solve_graph(tw_ctx* c, const HostGraph& g, int* tw_out, int32_t* order, int3
       fused_done = true;  // (no decide run and no walk)
     } else if (c->cfg.ub_shortcut && try_fused && fused_eligible(c, g)) {
       int status = 0, ans = -1, bail_k = -1;
-      rc = run_fused(c, g, kc, k0, g.n - 1, &R, &status, &ans, &bail_k, st, nullptr);
+      rc = run_fused(c, g, kc, k0, g.n - 1, &R, &status, &ans, &bail_k, st, nullptr, want_walk);
       if (rc) return rc;
       if (status == 1) {
         tw = ans;

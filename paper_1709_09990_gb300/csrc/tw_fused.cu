@@ -179,7 +179,7 @@ __device__ int group_decide(const FusedArgs<K>& a, int grp, unsigned int gb, uns
       // a run above a k that has answered (or given up) is not needed: one
       // thread looks and tells the group at the barrier
       if (gb == 0 && threadIdx.x == 0)
-        st->ctr[i + 1].pad[0] = k > *(volatile int*)&a.st[0]->settled_k ? 1u : 0u;
+        st->ctr[i + 1].pad[0] = k > kSettledBase - *(volatile int*)&a.st[0]->settled ? 1u : 0u;
       if (!barrier_wait(&st->arrive, round, nb, error, sSeen)) return -2;
       got = __ldcg(&st->ctr[i + 1].out_count);
       const unsigned int ovf = __ldcg(&st->ctr[i + 1].overflow);
@@ -256,7 +256,7 @@ __global__ void __launch_bounds__(kFusedWarps<K> * 32, 16 / kFusedWarps<K>)
       if (gb == 0 && threadIdx.x == 0) {
         a.st[grp]->result = result;
         a.st[grp]->run_last = last;
-        if (result == 1 || result == 2) atomicMin(&st0->settled_k, k);
+        if (result == 1 || result == 2) atomicMax(&st0->settled, kSettledBase - k);
       }
     }
     if (!barrier_wait(&st0->w_arrive, w_round, gridDim.x, &st0->error, &sSeen)) return;
@@ -365,15 +365,20 @@ cudaError_t launch_t(const FusedLaunch& f, cudaStream_t s) {
   a.order = f.order;
   a.parent = f.parent;
   a.bags = f.bags;
-  int dev = 0, sms = 0, per_sm = 0, coop = 0;
+  // 16 warps per SM; the grid is looked up once per thread and device
+  static thread_local int cached_dev = -1, grid = 0;
+  int dev = 0;
   cudaGetDevice(&dev);
-  cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
-  if (!coop) return cudaErrorNotSupported;
-  cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fused_solve_kernel<K>, kFusedWarps<K> * 32, 0);
-  if (per_sm < 1) return cudaErrorNotSupported;
-  // 16 warps per SM
-  const int grid = sms * std::min(per_sm, 16 / kFusedWarps<K>);
+  if (dev != cached_dev) {
+    int sms = 0, per_sm = 0, coop = 0;
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+    if (!coop) return cudaErrorNotSupported;
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, fused_solve_kernel<K>, kFusedWarps<K> * 32, 0);
+    if (per_sm < 1) return cudaErrorNotSupported;
+    grid = sms * std::min(per_sm, 16 / kFusedWarps<K>);
+    cached_dev = dev;
+  }
   if (grid < a.groups) return cudaErrorNotSupported;
   void* args[] = {&a};
   return cudaLaunchCooperativeKernel(reinterpret_cast<void*>(fused_solve_kernel<K>), dim3(grid),

@@ -52,6 +52,21 @@ int put_from_device(tw_ctx* c, void* dst, const void* src_dev, size_t bytes) {
   return TW_OK;
 }
 
+int fetch_solution(tw_ctx* c) {
+  SmallLayout L;
+  // the region order .. bags in one copy
+  constexpr size_t kRegion = SmallLayout().bounds - SmallLayout().order;
+  if (!c->h_out) {
+    if (cudaHostAlloc(reinterpret_cast<void**>(&c->h_out), kRegion, cudaHostAllocDefault) != cudaSuccess) {
+      c->h_out = nullptr;
+      cudaGetLastError();
+      return TW_ERR_CUDA;
+    }
+  }
+  TW_CK(cudaMemcpyAsync(c->h_out, small_at(c, L.order), kRegion, cudaMemcpyDeviceToHost, c->stream));
+  return TW_OK;
+}
+
 int put_solution(tw_ctx* c, int n, int words, int32_t* order, int32_t* td_parent, uint64_t* td_bags) {
   SmallLayout L;
   struct Part {
@@ -68,18 +83,12 @@ int put_solution(tw_ctx* c, int n, int words, int32_t* order, int32_t* td_parent
     else
       any_host = true;
   }
-  if (any_host) {
-    // the region order .. bags in one copy into the pinned mirror
-    constexpr size_t kRegion = SmallLayout().bounds - SmallLayout().order;
-    if (!c->h_out) {
-      if (cudaHostAlloc(reinterpret_cast<void**>(&c->h_out), kRegion, cudaHostAllocDefault) != cudaSuccess) {
-        c->h_out = nullptr;
-        cudaGetLastError();
-        return TW_ERR_CUDA;
-      }
-    }
-    TW_CK(cudaMemcpyAsync(c->h_out, small_at(c, L.order), kRegion, cudaMemcpyDeviceToHost, c->stream));
+  const bool fresh = any_host && c->h_out_fresh;  // (the fused solve has copied it already)
+  if (any_host && !fresh) {
+    const int rc = fetch_solution(c);
+    if (rc) return rc;
   }
+  c->h_out_fresh = false;
   TW_CK(cudaStreamSynchronize(c->stream));
   if (any_host)
     for (const Part& p : parts)
@@ -205,11 +214,22 @@ int load_graph(const uint64_t* adj, int n, HostGraph* g) {
 
 char* small_at(tw_ctx* c, size_t off) { return static_cast<char*>(c->small.ptr) + off; }
 
-// Uploads the adjacency in the key layout of class kc and in 64-bit rows.
+// Uploads the adjacency in the key layout of class kc and in 64-bit rows: one
+// copy of both from pinned memory.
 int upload_graph(tw_ctx* c, const HostGraph& g, KeyClass kc) {
   SmallLayout L;
-  std::vector<unsigned char> buf(TW_MAX_N * 16, 0);
+  if (!c->h_up) {
+    if (cudaHostAlloc(reinterpret_cast<void**>(&c->h_up), L.walk, cudaHostAllocDefault) != cudaSuccess) {
+      c->h_up = nullptr;
+      cudaGetLastError();
+      return TW_ERR_CUDA;
+    }
+    TW_CK(cudaEventCreateWithFlags(&c->ev_up, cudaEventDisableTiming));
+  } else {
+    TW_CK(cudaEventSynchronize(c->ev_up));
+  }
   const size_t w = key_bytes(kc);
+  unsigned char* buf = c->h_up + L.adj;
   for (int r = 0; r < g.n; ++r) {
     const uint64_t lo = g.rows[(size_t)r * g.words];
     const uint64_t hi = g.words > 1 ? g.rows[(size_t)r * g.words + 1] : 0;
@@ -223,8 +243,9 @@ int upload_graph(tw_ctx* c, const HostGraph& g, KeyClass kc) {
       std::memcpy(&buf[r * w + 8], &hi, 8);
     }
   }
-  TW_CK(cudaMemcpyAsync(small_at(c, L.adj), buf.data(), (size_t)g.n * w, cudaMemcpyHostToDevice, c->stream));
-  TW_CK(cudaMemcpyAsync(small_at(c, L.adj64), g.rows.data(), g.rows.size() * 8, cudaMemcpyHostToDevice, c->stream));
+  std::memcpy(c->h_up + L.adj64, g.rows.data(), g.rows.size() * 8);
+  TW_CK(cudaMemcpyAsync(small_at(c, L.adj), c->h_up, L.adj64 + g.rows.size() * 8, cudaMemcpyHostToDevice, c->stream));
+  TW_CK(cudaEventRecord(c->ev_up, c->stream));
   return TW_OK;
 }
 

@@ -102,6 +102,9 @@ struct tw_ctx {
   int fused_unit = 0;        // bytes per slot of its layout (8, or 16 for 128-bit states)
   bool fused_clean = false;  // every table slot of the fused buffer is empty
   FusedState* h_fused = nullptr;
+  bool h_out_fresh = false;        // h_out holds the solution of the solve under way
+  unsigned char* h_up = nullptr;   // pinned staging of upload_graph
+  cudaEvent_t ev_up = nullptr;     // after the last copy from h_up
   unsigned char* h_out = nullptr;  // pinned mirror of the small buffer's order .. bags region
   std::vector<unsigned long long> fused_skip;
   // options of Section 3.1 for the decide run being prepared
@@ -177,6 +180,9 @@ int put_from_device(tw_ctx* c, void* dst, const void* src_dev, size_t bytes);
 // The ordering, tree-decomposition parents and bags of a solve from the small
 // buffer into the caller's pointers (each host, device or NULL) with one
 // stream synchronisation.
+// Enqueues the copy of the small buffer's order .. bags region into the pinned
+// mirror h_out (allocated on first use).
+int fetch_solution(tw_ctx* c);
 int put_solution(tw_ctx* c, int n, int words, int32_t* order, int32_t* td_parent, uint64_t* td_bags);
 size_t total_bytes(const tw_ctx* c);
 int grow(tw_ctx* c, DevBuf* b, size_t need, size_t keep);

@@ -91,6 +91,10 @@ cudaError_t launch_bounds(const unsigned long long* adj, const int32_t* n, const
                           int num_graphs, int32_t* out, float* feats, cudaStream_t s,
                           int lower_only = 0);
 
+// The lower bounds alone of one graph (n rows of ceil(n/64) words): out[0], out[1];
+// out[2] = out[3] = -1.
+cudaError_t launch_lower_bounds(const unsigned long long* adj, int n, int32_t* out, cudaStream_t s);
+
 // ---- partitioned insert (tw_partition.cu) ----------------------------------
 constexpr int kMaxRanges = 64;
 
@@ -151,10 +155,11 @@ cudaError_t launch_graph_clear(KeyClass kc, const GraphState* st, void* table, c
 cudaError_t launch_graph_expand(const GraphState* st, const ExpandLaunch& base, cudaStream_t s);
 
 // ---- fused small solve (tw_fused.cu) -----------------------------------------
+constexpr int kSettledBase = 1 << 20;  // above every k
 constexpr int kFusedMaxGroups = 4;  // decide runs of the sweep in flight at once
 
 // Device state of one group of a fused solve (zeroed by the host before the
-// launch, but for settled_k).  Group 0's state also holds the solve's summary and the window
+// launch).  Group 0's state also holds the solve's summary and the window
 // barrier of the whole grid.
 struct FusedState {
   unsigned long long level_off[130];  // arena index of level j of the group's run
@@ -171,8 +176,8 @@ struct FusedState {
                                       // index of the final level of the deciding run and
                                       // the group that ran it
   int k_start;                        // group 0: the first k of the sweep
-  int settled_k;                      // group 0: the smallest k that answered yes or gave up
-                                      // (set to INT_MAX by the launch)
+  int settled;                        // group 0: kSettledBase minus the smallest k that answered
+                                      // yes or gave up (0: none yet)
 };
 
 struct FusedLaunch {
