@@ -29,7 +29,7 @@ __global__ void __launch_bounds__(kBatchWarps * 32, 6)
                         const unsigned long long* __restrict__ adj_all, unsigned long long* table,
                         unsigned long long* out_keys, uint32_t* out_parent, BatchCounters* ctr, int max_probes) {
   using K = unsigned long long;
-  __shared__ K sAdj[kBatchWarps][64];
+  __shared__ AdjRow<K> sAdj[kBatchWarps][64];
   __shared__ core::WarpScratch<K> sScratch[kBatchWarps];
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
@@ -62,8 +62,8 @@ __global__ void __launch_bounds__(kBatchWarps * 32, 6)
       sg = segs[cur];
       __syncwarp();
       const K* a = adj_all + (size_t)sg.graph * 64;
-      sAdj[warp][lane] = lane < sg.n ? a[lane] : 0ull;
-      sAdj[warp][lane + 32] = lane + 32 < sg.n ? a[lane + 32] : 0ull;
+      sAdj[warp][lane] = {lane < sg.n ? a[lane] : 0ull, kbit<K>(lane)};
+      sAdj[warp][lane + 32] = {lane + 32 < sg.n ? a[lane + 32] : 0ull, kbit<K>(lane + 32)};
       __syncwarp();
       valid = kfirst_n<K>(sg.n);
       out.keys = out_keys + sg.o_off;
@@ -80,7 +80,7 @@ __global__ void __launch_bounds__(kBatchWarps * 32, 6)
     core::Candidates<K> cand = core::start_chunk<K, true>(S, active, sAdj[warp], valid, valid, sg.n, sg.k, lane, w);
     out.parent_base = (uint32_t)(local * 32ull);
     do {
-      const int total = core::build_queue<K>(cand, lane, w);
+      const int total = core::build_queue<K>(cand, lane, sAdj[warp], w);
       generated += (unsigned long long)core::search_insert<K, true>(w, total, staged, lane, sAdj[warp], sg.k,
                                                                     table + sg.t_off, sg.t_slots, max_probes, out);
       __syncwarp();

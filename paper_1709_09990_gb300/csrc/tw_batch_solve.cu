@@ -77,7 +77,7 @@ __device__ void block_fingerprint(const K* keys, unsigned long long count, unsig
 // the levels outgrow the workspace; else *yes and *last (the final level).
 // With fp_sum / fp_xor (decide mode) the level fingerprints are written.
 template <int kWarps>
-__device__ __noinline__ bool block_decide(const BatchSolveArgs& a, const K* adj, int n, int k, Work& w, K* sAdj,
+__device__ __noinline__ bool block_decide(const BatchSolveArgs& a, const K* adj, int n, int k, Work& w, AdjRow<K>* sAdj,
                              core::WarpScratch<K>* sScratch, const unsigned long long* sSets,
                              unsigned long long* sRed, bool* yes, int* last,
                              unsigned long long* stats, unsigned long long* fp_sum, unsigned long long* fp_xor) {
@@ -176,7 +176,7 @@ __device__ __noinline__ bool block_decide(const BatchSolveArgs& a, const K* adj,
 
 template <int kWarps>
 __global__ void __launch_bounds__(kWarps * 32, 24 / kWarps) batch_solve_kernel(const BatchSolveArgs a) {
-  __shared__ K sAdj[64];
+  __shared__ AdjRow<K> sAdj[64];
   __shared__ core::WarpScratch<K> sScratch[kWarps];
   __shared__ unsigned long long sRed[2 * kWarps];
   __shared__ unsigned long long sSets[65];  // C(n, j), capped

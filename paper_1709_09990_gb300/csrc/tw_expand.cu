@@ -42,7 +42,7 @@ using core::kFull;
 template <class K, int kWarps, bool kMMW = false>
 __global__ void __launch_bounds__(kWarps * 32, ResidentWarps<K>::value / kWarps)
     expand_insert_kernel(const ExpandParams<K> p) {
-  __shared__ K sAdj[KeyTraits<K>::kBits];
+  __shared__ AdjRow<K> sAdj[KeyTraits<K>::kBits];
   __shared__ core::WarpScratch<K> sScratch[kWarps];
   core::expand_level<K, kWarps, kMMW>(p, sAdj, sScratch);
 }
@@ -52,7 +52,7 @@ __global__ void __launch_bounds__(kWarps * 32, ResidentWarps<K>::value / kWarps)
 template <class K>
 __global__ void __launch_bounds__(4 * 32, ResidentWarps<K>::value / 4)
     expand_ranged_kernel(const ExpandParams<K> p, K* out_tail, unsigned long long out_split) {
-  __shared__ K sAdj[KeyTraits<K>::kBits];
+  __shared__ AdjRow<K> sAdj[KeyTraits<K>::kBits];
   __shared__ core::WarpScratch<K> sScratch[4];
   core::expand_level<K, 4, false, true>(p, sAdj, sScratch, 0u, 0u, out_tail, out_split);
 }

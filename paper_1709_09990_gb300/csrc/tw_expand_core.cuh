@@ -34,16 +34,16 @@ __device__ __forceinline__ unsigned long long home_slot(unsigned long long h, un
 // (both empty for S = {}), by a bitset flood fill over the adjacency rows in
 // shared memory.
 template <class K>
-__device__ __forceinline__ void min_component(const K S, const K* __restrict__ sAdj, K& comp, K& bnd) {
+__device__ __forceinline__ void min_component(const K S, const AdjRow<K>* __restrict__ sAdj, K& comp, K& bnd) {
   comp = kzero<K>();
   K q = kzero<K>();
   K front = klsb(S);
   while (!kempty(front)) {
-    const K b = klsb(front);
-    const K r = sAdj[kindex(b)];
-    q |= r;
-    comp |= b;
-    front = (front | r) & S & ~comp;
+    K ub = kzero<K>();
+    const AdjRow<K> a = sAdj[pick(front, ub)];
+    q |= a.row;
+    comp |= bit_of(a, ub);
+    front = (front | a.row) & S & ~comp;
   }
   bnd = q & ~S;
 }
@@ -71,15 +71,17 @@ struct Candidates {
 };
 template <class K, bool kCanonical>
 __device__ __forceinline__ Candidates<K> cheap_candidates(const K S, const K comp0, const K b0,
-                                                          const K* __restrict__ sAdj, const K valid, const K allowed,
+                                                          const AdjRow<K>* __restrict__ sAdj, const K valid, const K allowed,
                                                           const int k) {
   K cand = valid & allowed & ~S;
   if (kCanonical) cand &= kbelow_lowest(S) | b0;
   Candidates<K> c{kzero<K>(), kzero<K>()};
   while (!kempty(cand)) {
-    const K vb = klsb(cand);
+    K vb = kzero<K>();
+    const AdjRow<K> a = sAdj[pick(cand, vb)];
+    vb = bit_of(a, vb);
+    const K nv = a.row;
     cand ^= vb;
-    const K nv = sAdj[kindex(vb)];
     K t = nv, visit = nv & S;
     int most = k;
     if (kCanonical && !kempty(b0 & vb)) {
@@ -102,12 +104,13 @@ __device__ __forceinline__ Candidates<K> cheap_candidates(const K S, const K com
 // whole component at once (comp0, boundary b0), visits the vertices of S
 // reachable from v and gathers their rows; it stops as soon as the vertices
 // gathered outside S u {v} exceed k.
+//
+// vb is v's bit, nv its row.
 template <class K>
-__device__ __forceinline__ bool extension_feasible(const K S, const K comp0, const K b0, const int v,
-                                                   const K* __restrict__ sAdj, const int k) {
-  const K vb = kbit<K>(v);
+__device__ __forceinline__ bool extension_feasible(const K S, const K comp0, const K b0, const K vb, const K nv,
+                                                   const AdjRow<K>* __restrict__ sAdj, const int k) {
   const K out = ~(S | vb);
-  K q = sAdj[v];
+  K q = nv;
   K done = ~S;  // vertices that need no visit: those outside S and those visited
   if (!kempty(b0 & vb)) {
     done |= comp0;
@@ -117,11 +120,11 @@ __device__ __forceinline__ bool extension_feasible(const K S, const K comp0, con
   bool within;
   // (one way out of the loop, so that the warp's lanes meet again after it)
   while ((within = kpopc(q & out) <= k) && !kempty(front)) {
-    const K b = klsb(front);
-    const K r = sAdj[kindex(b)];
-    q |= r;
-    done |= b;
-    front = (front | r) & ~done;
+    K ub = kzero<K>();
+    const AdjRow<K> a = sAdj[pick(front, ub)];
+    q |= a.row;
+    done |= bit_of(a, ub);
+    front = (front | a.row) & ~done;
   }
   return within;
 }
@@ -149,7 +152,7 @@ __device__ __forceinline__ void warp_min_pair(int& d, int& v) {
 // into its minimum-degree neighbour (lowest index).  With at most k+1
 // vertices left no degree can exceed k, so the answer is settled.
 template <class K>
-__device__ __forceinline__ bool mmw_exceeds(const K S, const K* __restrict__ sAdj, const int n, const int k,
+__device__ __forceinline__ bool mmw_exceeds(const K S, const AdjRow<K>* __restrict__ sAdj, const int n, const int k,
                                             const int lane) {
   constexpr int NV = KeyTraits<K>::kBits / 32;  // vertices per lane
   constexpr int kNone = 1 << 30;
@@ -160,14 +163,15 @@ __device__ __forceinline__ bool mmw_exceeds(const K S, const K* __restrict__ sAd
     const int v = lane + 32 * t;
     row[t] = kzero<K>();
     if (v < n && ktest(alive, v)) {
-      const K nv = sAdj[v];
+      const K nv = sAdj[v].row;
       K q = nv & ~S;
       K vis = nv & S;
       K front = vis;
       while (!kempty(front)) {
-        const K b = klsb(front);
-        front ^= b;
-        const K r = sAdj[kindex(b)];
+        K ub = kzero<K>();
+        const AdjRow<K> a = sAdj[pick(front, ub)];
+        front ^= bit_of(a, ub);
+        const K r = a.row;
         q |= r & ~S;
         const K nw = r & S & ~vis;
         vis |= nw;
@@ -238,7 +242,7 @@ __device__ __forceinline__ bool mmw_exceeds(const K S, const K* __restrict__ sAd
 // with a minor-min-width bound above k?  (The warp examines its states one by
 // one.)
 template <class K>
-__device__ __forceinline__ bool mmw_prunes(const K S, const bool extendable, const K* __restrict__ sAdj, const int n,
+__device__ __forceinline__ bool mmw_prunes(const K S, const bool extendable, const AdjRow<K>* __restrict__ sAdj, const int n,
                                            const int k, const int lane) {
   unsigned pending = __ballot_sync(kFull, extendable);
   bool mine = false;
@@ -265,13 +269,30 @@ struct WarpScratch {
   uint16_t queue[32 * kTake];
 };
 
+// Takes a vertex out of a non-empty set: by its row's bit for 64-bit sets (2%
+// faster there), as the lowest one for the others.
+template <class K>
+__device__ __forceinline__ int take_vertex(K& set, const AdjRow<K>*) {
+  const K b = klsb(set);
+  set ^= b;
+  return kindex(b);
+}
+template <>
+__device__ __forceinline__ int take_vertex<unsigned long long>(unsigned long long& set,
+                                                               const AdjRow<unsigned long long>* sAdj) {
+  const int v = khighest(set);
+  set ^= sAdj[v].bit;
+  return v;
+}
+
 // Packs up to kTake (S, v) pairs of each of the warp's 32 states into the
 // warp's queue (entry = lane << 8 | v) and takes them out of c; returns the
 // number of pairs (warp uniform).  The pairs that need no search come first, so
 // that the searches run in as few rounds of the warp as they fill (a round
 // takes as long as its longest search).
 template <class K>
-__device__ __forceinline__ int build_queue(Candidates<K>& c, const int lane, WarpScratch<K>& w) {
+__device__ __forceinline__ int build_queue(Candidates<K>& c, const int lane, const AdjRow<K>* __restrict__ sAdj,
+                                           WarpScratch<K>& w) {
   const int n0 = min(kpopc(c.done), kTake);
   const int n1 = min(kpopc(c.search), kTake - n0);
   const int cnt = n0 | (n1 << 16);
@@ -285,15 +306,13 @@ __device__ __forceinline__ int build_queue(Candidates<K>& c, const int lane, War
   const int excl = incl - cnt;
   int pos = excl & 0xffff;
   for (int end = pos + n0; pos < end; ++pos) {
-    const K vb = klsb(c.done);
-    c.done ^= vb;
-    w.queue[pos] = (uint16_t)((lane << 8) | kindex(vb));
+    const int v = take_vertex(c.done, sAdj);
+    w.queue[pos] = (uint16_t)((lane << 8) | v);
   }
   pos = (total & 0xffff) + (excl >> 16);
   for (int end = pos + n1; pos < end; ++pos) {
-    const K vb = klsb(c.search);
-    c.search ^= vb;
-    w.queue[pos] = (uint16_t)((lane << 8) | kindex(vb));
+    const int v = take_vertex(c.search, sAdj);
+    w.queue[pos] = (uint16_t)((lane << 8) | v);
   }
   __syncwarp();
   return (total & 0xffff) + (total >> 16);
@@ -307,7 +326,7 @@ __device__ __forceinline__ bool any_left(const Candidates<K>& c) {
 // test; returns the surviving candidates of this lane's state.  Inactive lanes
 // pass active = false.
 template <class K, bool kCanonical, bool kMMW = false>
-__device__ __forceinline__ Candidates<K> start_chunk(const K S, const bool active, const K* __restrict__ sAdj,
+__device__ __forceinline__ Candidates<K> start_chunk(const K S, const bool active, const AdjRow<K>* __restrict__ sAdj,
                                                      const K valid, const K allowed, const int n, const int k,
                                                      const int lane, WarpScratch<K>& w) {
   K comp0 = kzero<K>(), b0 = kzero<K>();
@@ -327,7 +346,7 @@ __device__ __forceinline__ Candidates<K> start_chunk(const K S, const bool activ
 // front of the queue; returns their number (warp uniform).
 template <class K>
 __device__ __forceinline__ int keep_feasible(WarpScratch<K>& w, const int total, const int lane,
-                                             const K* __restrict__ sAdj, const int k) {
+                                             const AdjRow<K>* __restrict__ sAdj, const int k) {
   int kept = 0;
   for (int base = 0; base < total; base += 32) {
     const int j = base + lane;
@@ -335,7 +354,9 @@ __device__ __forceinline__ int keep_feasible(WarpScratch<K>& w, const int total,
     bool ok = false;
     if (j < total) {
       e = w.queue[j];
-      ok = extension_feasible<K>(w.state[e >> 8], w.comp[e >> 8], w.bnd[e >> 8], e & 0xff, sAdj, k);
+      const AdjRow<K> av = sAdj[e & 0xff];
+      ok = extension_feasible<K>(w.state[e >> 8], w.comp[e >> 8], w.bnd[e >> 8], own_bit(av, e & 0xff), av.row, sAdj,
+                                 k);
     }
     const unsigned m = __ballot_sync(kFull, ok);  // (every lane has read its entry)
     if (ok) w.queue[kept + __popc(m & ((1u << lane) - 1u))] = e;
@@ -491,7 +512,7 @@ __device__ __forceinline__ bool insert_key(K* __restrict__ table, const unsigned
 // mod 2^64) * sectors).
 template <class K, bool kParent, bool kRanged = false>
 __device__ __forceinline__ int search_insert(WarpScratch<K>& w, const int total, int& staged, const int lane,
-                                             const K* __restrict__ sAdj, const int k, K* __restrict__ table,
+                                             const AdjRow<K>* __restrict__ sAdj, const int k, K* __restrict__ table,
                                              const unsigned long long slots, const int max_probes,
                                              const LevelOut<K, kParent>& out, const unsigned long long ranges = 1,
                                              const unsigned long long range = 0, K* tail = nullptr,
@@ -505,8 +526,10 @@ __device__ __forceinline__ int search_insert(WarpScratch<K>& w, const int total,
     const bool have = base + lane < total;
     const int e = have ? w.queue[base + lane] : 0;
     const K S = w.state[e >> 8];
-    const K key = S | kbit<K>(e & 0xff);
-    bool ok = have && extension_feasible<K>(S, w.comp[e >> 8], w.bnd[e >> 8], e & 0xff, sAdj, k);
+    const AdjRow<K> av = sAdj[e & 0xff];
+    const K vb = own_bit(av, e & 0xff);
+    const K key = S | vb;
+    bool ok = have && extension_feasible<K>(S, w.comp[e >> 8], w.bnd[e >> 8], vb, av.row, sAdj, k);
     unsigned int home;
     if (kRanged) {
       const unsigned long long hash = khash(key);
@@ -643,11 +666,11 @@ __device__ __forceinline__ void add_warp_count(unsigned long long count, const i
 constexpr unsigned kSpreadWarps = 1024;
 template <class K, int kWarps, bool kMMW = false, bool kRanged = false, bool kBlockLocal = false,
           bool kKeysL2 = false, bool kGroup = false, bool kParent = false>
-__device__ __forceinline__ void expand_level(const ExpandParams<K>& p, K* sAdj, WarpScratch<K>* scratch,
+__device__ __forceinline__ void expand_level(const ExpandParams<K>& p, AdjRow<K>* sAdj, WarpScratch<K>* scratch,
                                              const unsigned group_block = 0, const unsigned group_blocks = 0,
                                              K* out_tail = nullptr, const unsigned long long out_split = 0) {
   if (!kGroup) {
-    for (int i = threadIdx.x; i < p.n; i += blockDim.x) sAdj[i] = p.adj[i];
+    for (int i = threadIdx.x; i < p.n; i += blockDim.x) set_row(sAdj[i], p.adj[i], i);
     __syncthreads();
   }
   const int lane = threadIdx.x & 31;
@@ -680,7 +703,7 @@ __device__ __forceinline__ void expand_level(const ExpandParams<K>& p, K* sAdj, 
     // feasible vertex)
     Candidates<K> c = start_chunk<K, !kMMW, kMMW>(S, active, sAdj, valid, p.allowed, p.n, p.k, lane, w);
     do {
-      const int total = build_queue<K>(c, lane, w);
+      const int total = build_queue<K>(c, lane, sAdj, w);
       generated += (unsigned long long)search_insert<K, kParent, kRanged>(w, total, staged, lane, sAdj, p.k, p.table,
                                                                            p.table_slots, p.max_probes, out, p.ranges,
                                                                            p.range, out_tail, out_split);

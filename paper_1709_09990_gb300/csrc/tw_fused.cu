@@ -113,7 +113,7 @@ struct FusedArgs {
 // index of the final level built.
 template <class K>
 __device__ int group_decide(const FusedArgs<K>& a, int grp, unsigned int gb, unsigned int nb, int k,
-                            unsigned long long dirty[2], int* last, K* sAdj, core::WarpScratch<K>* sScratch,
+                            unsigned long long dirty[2], int* last, AdjRow<K>* sAdj, core::WarpScratch<K>* sScratch,
                             const unsigned long long* sSets, unsigned int& round, unsigned int* sSeen) {
   FusedState* st = a.st[grp];
   unsigned int* error = &a.st[0]->error;
@@ -224,13 +224,13 @@ __device__ int group_decide(const FusedArgs<K>& a, int grp, unsigned int gb, uns
 template <class K>
 __global__ void __launch_bounds__(kFusedWarps<K> * 32, 16 / kFusedWarps<K>)
     fused_solve_kernel(const FusedArgs<K> a) {
-  __shared__ K sAdj[KeyTraits<K>::kBits];
+  __shared__ AdjRow<K> sAdj[KeyTraits<K>::kBits];
   __shared__ core::WarpScratch<K> sScratch[kFusedWarps<K>];
   __shared__ unsigned long long sSets[129];  // C(n, j), capped
   __shared__ unsigned int sSeen;
   __shared__ K128 sTdAdj[128];
   __shared__ int sPos[128];
-  for (int i = threadIdx.x; i < a.n; i += blockDim.x) sAdj[i] = a.adj[i];
+  for (int i = threadIdx.x; i < a.n; i += blockDim.x) set_row(sAdj[i], a.adj[i], i);
   for (int j = threadIdx.x; j <= a.n; j += blockDim.x) sSets[j] = core::binom_capped(a.n, j, core::kSetsCap);
   __syncthreads();
   unsigned int round = 0, w_round = 0;  // this block's barriers on its group's and the grid's counter

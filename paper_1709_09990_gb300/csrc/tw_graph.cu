@@ -93,7 +93,7 @@ __global__ void graph_clear_kernel(const GraphState* __restrict__ st, uint4* __r
 template <class K, int kWarps, bool kMMW>
 __global__ void __launch_bounds__(kWarps * 32, ResidentWarps<K>::value / kWarps)
     graph_expand_kernel(const GraphState* __restrict__ st, const ExpandParams<K> base) {
-  __shared__ K sAdj[KeyTraits<K>::kBits];
+  __shared__ AdjRow<K> sAdj[KeyTraits<K>::kBits];
   __shared__ core::WarpScratch<K> sScratch[kWarps];
   if (st->done || st->bail) return;
   ExpandParams<K> p = base;

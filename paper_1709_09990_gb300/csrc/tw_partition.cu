@@ -86,13 +86,13 @@ __global__ void __launch_bounds__(kWarps * 32, 6)
     emit_kernel(const ExpandParams<K> p, int P, K* __restrict__ cand_key, uint8_t* __restrict__ cand_v,
                 unsigned long long region_cap, unsigned long long* __restrict__ region_cnt,
                 unsigned int* __restrict__ overflow) {
-  __shared__ K sAdj[KeyTraits<K>::kBits];
+  __shared__ AdjRow<K> sAdj[KeyTraits<K>::kBits];
   __shared__ core::WarpScratch<K> sScratch[kWarps];
   __shared__ int sTotal[kWarps];
   __shared__ int sHist[kMaxRanges];
   __shared__ int sCursor[kMaxRanges];
   __shared__ unsigned long long sBase[kMaxRanges];
-  for (int i = threadIdx.x; i < p.n; i += blockDim.x) sAdj[i] = p.adj[i];
+  for (int i = threadIdx.x; i < p.n; i += blockDim.x) set_row(sAdj[i], p.adj[i], i);
   __syncthreads();
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
@@ -108,7 +108,7 @@ __global__ void __launch_bounds__(kWarps * 32, 6)
         p.mmw ? core::start_chunk<K, false, true>(S, active, sAdj, valid, p.allowed, p.n, p.k, lane, ws)
               : core::start_chunk<K, true>(S, active, sAdj, valid, p.allowed, p.n, p.k, lane, ws);
     do {
-      const int total = core::keep_feasible<K>(ws, core::build_queue<K>(c, lane, ws), lane, sAdj, p.k);
+      const int total = core::keep_feasible<K>(ws, core::build_queue<K>(c, lane, sAdj, ws), lane, sAdj, p.k);
       if (lane == 0) sTotal[warp] = total;
       for (int r = threadIdx.x; r < P; r += blockDim.x) sHist[r] = 0;
       __syncthreads();
