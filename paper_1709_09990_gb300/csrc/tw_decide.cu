@@ -690,6 +690,28 @@ int run_decide(tw_ctx* c, KeyClass kc, int n, int k, bool keep_levels, DecideRes
   return TW_OK;
 }
 
+// Fingerprints of levels 1 .. last of a run whose levels are all in one arena
+// (offsets and counts in device memory, and the counts here): one launch and
+// one copy back.
+int level_fingerprints(tw_ctx* c, KeyClass kc, const void* keys, const unsigned long long* d_off,
+                       const unsigned long long* d_cnt, const unsigned long long* cnt, int last, DecideResult* R) {
+  if (last < 1) return TW_OK;
+  SmallLayout L;
+  unsigned long long* d_out = reinterpret_cast<unsigned long long*>(small_at(c, L.fps));
+  unsigned long long most = 0;
+  for (int j = 1; j <= last; ++j) most = std::max(most, cnt[j]);
+  std::vector<unsigned long long> h(2 * (size_t)last);
+  TW_CK(cudaMemsetAsync(d_out, 0, h.size() * 8, c->stream));
+  TW_LAUNCH(c, launch_fingerprint_levels(kc, keys, d_off, d_cnt, last, most, d_out, c->stream));
+  TW_CK(cudaMemcpyAsync(h.data(), d_out, h.size() * 8, cudaMemcpyDeviceToHost, c->stream));
+  TW_CK(cudaStreamSynchronize(c->stream));
+  for (int j = 0; j < last; ++j) {
+    R->fp_sum.push_back(h[2 * j]);
+    R->fp_xor.push_back(h[2 * j + 1]);
+  }
+  return TW_OK;
+}
+
 // decide(k) with the level loop as one captured CUDA graph (every level kept).
 // *bailed is set when the graph gave up (a level did not fit the current
 // buffers or its estimate); the caller then runs the host loop.
@@ -827,17 +849,9 @@ int run_decide_graph(tw_ctx* c, KeyClass kc, int n, int k, DecideResult* R, bool
     }
   R->peak_bytes = h.peak_bytes;
   R->yes = h.yes;
-  if (c->cfg.fingerprints) {
-    for (int j = 1; j <= h.cur; ++j) {
-      TW_CK(cudaMemsetAsync(c->d_ctr, 0, sizeof(LevelCounters), c->stream));
-      TW_LAUNCH(c, launch_fingerprint(kc, static_cast<char*>(c->keys.ptr) + h.level_off[j] * w, h.level_cnt[j],
-                                      c->d_ctr, c->stream));
-      TW_CK(cudaMemcpyAsync(c->h_ctr, c->d_ctr, sizeof(LevelCounters), cudaMemcpyDeviceToHost, c->stream));
-      TW_CK(cudaStreamSynchronize(c->stream));
-      R->fp_sum.push_back(c->h_ctr->fp_sum);
-      R->fp_xor.push_back(c->h_ctr->fp_xor);
-    }
-  }
+  if (c->cfg.fingerprints)
+    return level_fingerprints(c, kc, c->keys.ptr, c->d_gstate->level_off, c->d_gstate->level_cnt, h.level_cnt, h.cur,
+                              R);
   return TW_OK;
 }
 
@@ -1184,15 +1198,9 @@ int run_fused(tw_ctx* c, const HostGraph& g, KeyClass kc, int k0, int k_last, De
   R->fp_sum.assign(1, 0ull);
   R->fp_xor.assign(1, 0ull);
   if (c->cfg.fingerprints) {
-    for (int j = 1; j <= h.last; ++j) {
-      TW_CK(cudaMemsetAsync(c->d_ctr, 0, sizeof(LevelCounters), c->stream));
-      TW_LAUNCH(c, launch_fingerprint(kc, static_cast<char*>(f.keys[grp]) + hl->level_off[j] * w, hl->level_cnt[j],
-                                      c->d_ctr, c->stream));
-      TW_CK(cudaMemcpyAsync(c->h_ctr, c->d_ctr, sizeof(LevelCounters), cudaMemcpyDeviceToHost, c->stream));
-      TW_CK(cudaStreamSynchronize(c->stream));
-      R->fp_sum.push_back(c->h_ctr->fp_sum);
-      R->fp_xor.push_back(c->h_ctr->fp_xor);
-    }
+    const int rc = level_fingerprints(c, kc, f.keys[grp], f.st[grp]->level_off, f.st[grp]->level_cnt, hl->level_cnt,
+                                      h.last, R);
+    if (rc) return rc;
   }
   fill_stats(*R, last_k, st, false);
   if (st) st->decide_runs += (unsigned long long)(last_k - k0);  // fill_stats counted one run

@@ -196,6 +196,32 @@ __global__ void fingerprint_kernel(const K* __restrict__ keys, unsigned long lon
   }
 }
 
+// The levels of a finished run in one launch: blockIdx.y + 1 is the level, whose
+// count keys lie at off; out[2 y], out[2 y + 1] += sum and xor.
+template <class K>
+__global__ void fingerprint_levels_kernel(const K* __restrict__ keys, const unsigned long long* __restrict__ off,
+                                          const unsigned long long* __restrict__ cnt, unsigned long long* out) {
+  const int level = blockIdx.y + 1;
+  const K* first = keys + off[level];
+  const unsigned long long count = cnt[level];
+  unsigned long long s = 0, x = 0;
+  const unsigned long long stride = (unsigned long long)gridDim.x * blockDim.x;
+  for (unsigned long long i = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; i < count; i += stride) {
+    const unsigned long long f = kfingerprint(first[i]);
+    s += f;
+    x ^= f;
+  }
+#pragma unroll
+  for (int d = 16; d > 0; d >>= 1) {
+    s += __shfl_xor_sync(kFull, s, d);
+    x ^= __shfl_xor_sync(kFull, x, d);
+  }
+  if ((threadIdx.x & 31) == 0 && (s | x)) {
+    atomicAdd(&out[2 * blockIdx.y], s);
+    atomicXor(&out[2 * blockIdx.y + 1], x);
+  }
+}
+
 // ------------------------------------------------------------ backward walk
 template <class K>
 __global__ void walk_init_kernel(const K* keys, K* walk, int last) {
@@ -279,6 +305,22 @@ cudaError_t launch_fingerprint(KeyClass kc, const void* keys, unsigned long long
       fingerprint_kernel<unsigned long long><<<g, 256, 0, s>>>(static_cast<const unsigned long long*>(keys), count, ctr);
       break;
     default: fingerprint_kernel<K128><<<g, 256, 0, s>>>(static_cast<const K128*>(keys), count, ctr); break;
+  }
+  return cudaGetLastError();
+}
+
+cudaError_t launch_fingerprint_levels(KeyClass kc, const void* keys, const unsigned long long* off,
+                                      const unsigned long long* cnt, int levels, unsigned long long most,
+                                      unsigned long long* out, cudaStream_t s) {
+  if (levels <= 0) return cudaSuccess;
+  const dim3 g((unsigned)stream_grid(most > 0 ? most : 1, 256 * 4), (unsigned)levels);
+  switch (kc) {
+    case kKey32: fingerprint_levels_kernel<uint32_t><<<g, 256, 0, s>>>(static_cast<const uint32_t*>(keys), off, cnt, out); break;
+    case kKey64:
+      fingerprint_levels_kernel<unsigned long long><<<g, 256, 0, s>>>(static_cast<const unsigned long long*>(keys), off,
+                                                                      cnt, out);
+      break;
+    default: fingerprint_levels_kernel<K128><<<g, 256, 0, s>>>(static_cast<const K128*>(keys), off, cnt, out); break;
   }
   return cudaGetLastError();
 }

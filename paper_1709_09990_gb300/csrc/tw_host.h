@@ -152,6 +152,7 @@ struct SmallLayout {
   size_t parent = 8704; // TW_MAX_N int32
   size_t bags = 9216;   // TW_MAX_N * 2 uint64
   size_t bounds = 11264;// 4 int32
+  size_t fps = 16384;   // 2 uint64 per level (TW_MAX_N + 1 levels)
 };
 
 struct LevelRec {

@@ -64,6 +64,13 @@ cudaError_t launch_widen32(const uint32_t* src, unsigned long long* dst, unsigne
 cudaError_t launch_fingerprint(KeyClass kc, const void* keys, unsigned long long count,
                                LevelCounters* ctr, cudaStream_t s);
 
+// out[2 j], out[2 j + 1] += sum and xor of the fingerprints of level j + 1, j <
+// levels: the cnt[j + 1] keys from off[j + 1] on (off, cnt: device arrays; the
+// largest count is `most`).  out zeroed by the caller.
+cudaError_t launch_fingerprint_levels(KeyClass kc, const void* keys, const unsigned long long* off,
+                                      const unsigned long long* cnt, int levels, unsigned long long most,
+                                      unsigned long long* out, cudaStream_t s);
+
 // One step of the backward walk: finds walk[j] among the count keys of level
 // j, writes its predecessor vertex v to order[j-1] and walk[j-1] = walk[j]
 // minus v.  walk holds one key per level.
