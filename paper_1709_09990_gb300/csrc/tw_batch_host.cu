@@ -27,7 +27,7 @@ constexpr int kBatchProbes = 256;
 // States that one block of copy_segments_kernel moves: levels are copied in
 // pieces of this size, so that a level of a million sets takes the whole GPU
 // and not one block (the copies of a 512-graph batch took 137 of its 371 ms).
-constexpr unsigned long long kCopyPiece = 8192;
+constexpr unsigned long long kCopyPiece = 4096;
 
 void add_copy(std::vector<CopySeg>* list, unsigned long long src, unsigned long long dst, unsigned long long count) {
   for (unsigned long long at = 0; at < count; at += kCopyPiece)
@@ -353,8 +353,9 @@ int run_batch(tw_ctx* c, const std::vector<HostGraph>& graphs, const std::vector
       TW_CK(cudaMemcpyAsync(B.walks, walks.data(), walks.size() * sizeof(WalkSeg), cudaMemcpyHostToDevice,
                             c->stream));
       TW_CK(cudaMemcpyAsync(B.lvl, lvl.data(), lvl.size() * 8, cudaMemcpyHostToDevice, c->stream));
+      // (not waited for: the levels it reads stay in the arena until later work of
+      // this stream)
       TW_LAUNCH(c, launch_walk_batch(B.walks, (int)walks.size(), B.lvl, B.akeys, B.apar, B.orders, c->stream));
-      TW_CK(cudaStreamSynchronize(c->stream));
       for (int j : walked) {
         record_answer(B.g[j], true);
         B.g[j].levels.clear();
