@@ -23,33 +23,76 @@ namespace {
 using core::kFull;
 constexpr int kBatchWarps = 4;
 
-// A warp's chunks are a grid apart (four in a row, to change graph less often,
-// made a 512-graph batch 40% slower); 32 warps per SM (24: 3% slower).
+// One graph's part of a warp's scratch: rows, states, queue and stage for sets
+// of type K (graphs of up to 32 vertices work on 32-bit sets and tables: half
+// the instructions and half the table; their lists hold 64-bit keys like the
+// others').
+template <class K>
+struct WarpGraph {
+  AdjRow<K> adj[KeyTraits<K>::kBits];
+  core::WarpScratch<K> w;
+};
+
+// A warp's chunk of 32 states of one graph.
+template <class K>
+__device__ __forceinline__ int expand_chunk(WarpGraph<K>& m, const unsigned long long key, const bool active,
+                                            const BatchSeg& sg, const int lane, int& staged, void* table,
+                                            const int max_probes,
+                                            const core::LevelOut<K, true, unsigned long long>& out) {
+  const K valid = kfirst_n<K>(sg.n);
+  int pairs = 0;
+  core::Candidates<K> cand =
+      core::start_chunk<K, true>(active ? (K)key : valid, active, m.adj, valid, valid, sg.n, sg.k, lane, m.w);
+  do {
+    const int total = core::build_queue<K>(cand, lane, m.adj, m.w);
+    pairs += core::search_insert<K, true, false, unsigned long long>(m.w, total, staged, lane, m.adj, sg.k,
+                                                                     static_cast<K*>(table), sg.t_slots, max_probes,
+                                                                     out);
+    __syncwarp();
+  } while (__any_sync(kFull, core::any_left(cand)));
+  return pairs;
+}
+
+// A warp's first chunk is its own number, the others come from a counter (one
+// add per chunk, on its way while the chunk before is worked on): the chunks of
+// a batch cost between one and ten times the same, and with fixed shares the
+// slowest SM took 1.5 times the average.  32 warps per SM (24: 3% slower).
 __global__ void __launch_bounds__(kBatchWarps * 32, 8)
     expand_batch_kernel(const BatchSeg* __restrict__ segs, const unsigned long long* __restrict__ chunk_begin,
                         int nseg, unsigned long long total_chunks, const unsigned long long* __restrict__ keys,
                         const unsigned long long* __restrict__ adj_all, unsigned long long* table,
                         unsigned long long* out_keys, uint32_t* out_parent, BatchCounters* ctr, int max_probes) {
-  using K = unsigned long long;
-  __shared__ AdjRow<K> sAdj[kBatchWarps][64];
-  __shared__ core::WarpScratch<K> sScratch[kBatchWarps];
+  using K64 = unsigned long long;
+  union Mine {
+    WarpGraph<K64> wide;
+    WarpGraph<uint32_t> narrow;
+    __device__ Mine() {}
+  };
+  __shared__ __align__(16) unsigned char sMine[kBatchWarps][sizeof(Mine)];
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
+  Mine& m = *reinterpret_cast<Mine*>(sMine[warp]);
   const unsigned long long stride = (unsigned long long)gridDim.x * kBatchWarps;
   int cur = -1;
+  bool narrow = false;
   BatchSeg sg{};
-  K valid = 0;
-  core::LevelOut<K, true> out{};
-  core::WarpScratch<K>& w = sScratch[warp];
+  core::LevelOut<K64, true, K64> wide_out{};
+  core::LevelOut<uint32_t, true, K64> narrow_out{};
   int staged = 0;
   unsigned long long generated = 0;
   // the warp's staged sets and pair count go to its graph's list and counter
   auto finish_graph = [&]() {
-    core::flush_stage<K, true, false>(w, staged, lane, out, nullptr, 0ull);
+    if (narrow)
+      core::flush_stage<uint32_t, true, false, K64>(m.narrow.w, staged, lane, narrow_out, nullptr, 0ull);
+    else
+      core::flush_stage<K64, true, false, K64>(m.wide.w, staged, lane, wide_out, nullptr, 0ull);
     core::add_warp_count(generated, lane, &ctr[cur].generated);
     generated = 0;
   };
-  for (unsigned long long c = (unsigned long long)blockIdx.x * kBatchWarps + warp; c < total_chunks; c += stride) {
+  unsigned long long* next_chunk = &ctr[nseg].out_count;  // (zero at the launch)
+  for (unsigned long long c = (unsigned long long)blockIdx.x * kBatchWarps + warp; c < total_chunks;) {
+    unsigned long long next = 0;
+    if (lane == 0) next = stride + atomicAdd(next_chunk, 1ull);
     if (cur < 0 || c < chunk_begin[cur] || c >= chunk_begin[cur + 1]) {
       if (cur >= 0) finish_graph();
       int lo = 0, hi = nseg - 1;  // last s with chunk_begin[s] <= c
@@ -62,31 +105,36 @@ __global__ void __launch_bounds__(kBatchWarps * 32, 8)
       }
       cur = lo;
       sg = segs[cur];
+      narrow = sg.n <= 32;
       __syncwarp();
-      const K* a = adj_all + (size_t)sg.graph * 64;
-      sAdj[warp][lane] = {lane < sg.n ? a[lane] : 0ull, kbit<K>(lane)};
-      sAdj[warp][lane + 32] = {lane + 32 < sg.n ? a[lane + 32] : 0ull, kbit<K>(lane + 32)};
+      const K64* a = adj_all + (size_t)sg.graph * 64;
+      if (narrow) {
+        set_row(m.narrow.adj[lane], lane < sg.n ? (uint32_t)a[lane] : 0u, lane);
+      } else {
+        set_row(m.wide.adj[lane], lane < sg.n ? a[lane] : 0ull, lane);
+        set_row(m.wide.adj[lane + 32], lane + 32 < sg.n ? a[lane + 32] : 0ull, lane + 32);
+      }
       __syncwarp();
-      valid = kfirst_n<K>(sg.n);
-      out.keys = out_keys + sg.o_off;
-      out.pred = nullptr;
-      out.parent = out_parent + sg.o_off;
-      out.cap = sg.o_cap;
-      out.count = &ctr[cur].out_count;
-      out.overflow = &ctr[cur].overflow;
+      wide_out.keys = narrow_out.keys = out_keys + sg.o_off;
+      wide_out.parent = narrow_out.parent = out_parent + sg.o_off;
+      wide_out.cap = narrow_out.cap = sg.o_cap;
+      wide_out.count = narrow_out.count = &ctr[cur].out_count;
+      wide_out.overflow = narrow_out.overflow = &ctr[cur].overflow;
     }
     const unsigned long long local = c - chunk_begin[cur];
     const unsigned long long idx = local * 32ull + lane;
     const bool active = idx < sg.in_count;
-    const K S = active ? keys[sg.in_off + idx] : valid;
-    core::Candidates<K> cand = core::start_chunk<K, true>(S, active, sAdj[warp], valid, valid, sg.n, sg.k, lane, w);
-    out.parent_base = (uint32_t)(local * 32ull);
-    do {
-      const int total = core::build_queue<K>(cand, lane, sAdj[warp], w);
-      generated += (unsigned long long)core::search_insert<K, true>(w, total, staged, lane, sAdj[warp], sg.k,
-                                                                    table + sg.t_off, sg.t_slots, max_probes, out);
-      __syncwarp();
-    } while (__any_sync(kFull, core::any_left(cand)));
+    const K64 key = active ? keys[sg.in_off + idx] : 0ull;
+    if (narrow) {
+      narrow_out.parent_base = (uint32_t)(local * 32ull);
+      generated += (unsigned long long)expand_chunk<uint32_t>(m.narrow, key, active, sg, lane, staged,
+                                                              table + sg.t_off, max_probes, narrow_out);
+    } else {
+      wide_out.parent_base = (uint32_t)(local * 32ull);
+      generated += (unsigned long long)expand_chunk<K64>(m.wide, key, active, sg, lane, staged, table + sg.t_off,
+                                                         max_probes, wide_out);
+    }
+    c = __shfl_sync(kFull, next, 0);
   }
   if (cur >= 0) finish_graph();
 }

@@ -246,7 +246,7 @@ int run_batch(tw_ctx* c, const std::vector<HostGraph>& graphs, const std::vector
   // (a step's pieces: its segments' last ones and the whole ones of its output;
   // grown below if a step ever has more)
   size_t copy_room = (size_t)G + (size_t)(kStepOut / kCopyPiece) + 1024;
-  if ((rc = dev_alloc(&B.segs, G)) || (rc = dev_alloc(&B.cbeg, (size_t)G + 1)) || (rc = dev_alloc(&B.ctr, G)) ||
+  if ((rc = dev_alloc(&B.segs, G)) || (rc = dev_alloc(&B.cbeg, (size_t)G + 1)) || (rc = dev_alloc(&B.ctr, (size_t)G + 1)) ||
       (rc = dev_alloc(&B.copies, copy_room)) || (rc = dev_alloc(&B.walks, G)) ||
       (rc = dev_alloc(&B.lvl, (size_t)G * 65)))
     return rc;
@@ -435,7 +435,8 @@ int run_batch(tw_ctx* c, const std::vector<HostGraph>& graphs, const std::vector
     const int nseg = (int)segs.size();
     TW_CK(cudaMemcpyAsync(B.segs, segs.data(), nseg * sizeof(BatchSeg), cudaMemcpyHostToDevice, c->stream));
     TW_CK(cudaMemcpyAsync(B.cbeg, cbeg.data(), (nseg + 1) * 8, cudaMemcpyHostToDevice, c->stream));
-    TW_CK(cudaMemsetAsync(B.ctr, 0, nseg * sizeof(BatchCounters), c->stream));
+    // (one more: the chunk counter of the launch)
+    TW_CK(cudaMemsetAsync(B.ctr, 0, (nseg + 1) * sizeof(BatchCounters), c->stream));
     TW_LAUNCH(c, launch_clear(B.table, (size_t)((tsum * 8 + 15) & ~15ull), c->d_ctr, c->stream));
     TW_LAUNCH(c, launch_expand_batch(B.segs, B.cbeg, nseg, chunks, B.akeys, B.adj, B.table, B.okeys, B.opar, B.ctr,
                                      kBatchProbes, c->stream));

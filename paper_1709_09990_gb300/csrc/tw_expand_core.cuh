@@ -369,9 +369,11 @@ __device__ __forceinline__ int keep_feasible(WarpScratch<K>& w, const int total,
 // Where the winners of the inserts go.  With kParent the output records the
 // index (parent_base + lane) of the parent state in its level; otherwise the
 // added vertex.
-template <class K, bool kParent>
+// KO is the type of the list's keys (wider than the search's in the batched
+// kernel, whose lists hold 64-bit keys).
+template <class K, bool kParent, class KO = K>
 struct LevelOut {
-  K* keys;
+  KO* keys;
   uint8_t* pred;       // used when !kParent
   uint32_t* parent;    // used when kParent
   uint32_t parent_base;
@@ -384,9 +386,9 @@ struct LevelOut {
 // kRanged no predecessor is stored and output positions from split on go to
 // tail[position - split] when tail is given (a list continued in a second
 // buffer).
-template <class K, bool kParent, bool kRanged>
+template <class K, bool kParent, bool kRanged, class KO = K>
 __device__ __forceinline__ void store_stage(const WarpScratch<K>& w, const int staged, const unsigned long long b,
-                                            const int lane, const LevelOut<K, kParent>& out, K* tail,
+                                            const int lane, const LevelOut<K, kParent, KO>& out, K* tail,
                                             const unsigned long long split) {
   for (int j = lane; j < staged; j += 32) {
     const unsigned long long o = b + (unsigned long long)j;
@@ -394,7 +396,7 @@ __device__ __forceinline__ void store_stage(const WarpScratch<K>& w, const int s
       if (kRanged && tail != nullptr && o >= split)
         kstore_cs(&tail[o - split], w.stage_key[j]);
       else
-        kstore_cs(&out.keys[o], w.stage_key[j]);
+        kstore_cs(&out.keys[o], (KO)w.stage_key[j]);
       if (kParent)
         __stcs(&out.parent[o], w.stage_from[j]);
       else if (!kRanged)
@@ -409,15 +411,15 @@ __device__ __forceinline__ void store_stage(const WarpScratch<K>& w, const int s
 // them.  (Every add of a level goes to the same counter, which takes about one
 // in 2.6 ns; with one add per 64 pairs that was the whole time of a level, with
 // one per 200 new sets it no longer shows.)
-template <class K, bool kParent, bool kRanged>
+template <class K, bool kParent, bool kRanged, class KO = K>
 __device__ __forceinline__ void flush_stage(WarpScratch<K>& w, int& staged, const int lane,
-                                            const LevelOut<K, kParent>& out, K* tail, const unsigned long long split) {
+                                            const LevelOut<K, kParent, KO>& out, K* tail, const unsigned long long split) {
   if (staged == 0) return;
   __syncwarp();
   unsigned long long b = 0;
   if (lane == 0) b = atomicAdd(out.count, (unsigned long long)staged);
   b = __shfl_sync(kFull, b, 0);
-  store_stage<K, kParent, kRanged>(w, staged, b, lane, out, tail, split);
+  store_stage<K, kParent, kRanged, KO>(w, staged, b, lane, out, tail, split);
   staged = 0;
   __syncwarp();
 }
@@ -510,11 +512,11 @@ __device__ __forceinline__ bool insert_key(K* __restrict__ table, const unsigned
 // pairs of one of the ranges); the table is the slice of that range (the home
 // spreads the range's hashes over the slice: the high word of (hash * ranges
 // mod 2^64) * sectors).
-template <class K, bool kParent, bool kRanged = false>
+template <class K, bool kParent, bool kRanged = false, class KO = K>
 __device__ __forceinline__ int search_insert(WarpScratch<K>& w, const int total, int& staged, const int lane,
                                              const AdjRow<K>* __restrict__ sAdj, const int k, K* __restrict__ table,
                                              const unsigned long long slots, const int max_probes,
-                                             const LevelOut<K, kParent>& out, const unsigned long long ranges = 1,
+                                             const LevelOut<K, kParent, KO>& out, const unsigned long long ranges = 1,
                                              const unsigned long long range = 0, K* tail = nullptr,
                                              const unsigned long long split = 0) {
   constexpr int B = Sector<K>::kSlots;
@@ -544,7 +546,7 @@ __device__ __forceinline__ int search_insert(WarpScratch<K>& w, const int total,
     __syncwarp();
     const bool won = ok && insert_key<K>(table, sectors, max_sectors, home, key, out.overflow);
     __syncwarp();
-    if (staged > kStage - 32) flush_stage<K, kParent, kRanged>(w, staged, lane, out, tail, split);
+    if (staged > kStage - 32) flush_stage<K, kParent, kRanged, KO>(w, staged, lane, out, tail, split);
     const unsigned wm = __ballot_sync(kFull, won);
     if (won) {
       const int o = staged + __popc(wm & ((1u << lane) - 1u));

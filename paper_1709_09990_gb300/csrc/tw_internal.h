@@ -288,7 +288,8 @@ struct WalkSeg {
 };
 
 // chunk_begin has nseg+1 entries (the last one = total_chunks); segments
-// must be non-empty.  Keys are u64, parents u32.
+// must be non-empty.  ctr has nseg+1 zeroed entries (the last one: the launch's
+// chunk counter).  Keys are u64, parents u32.
 cudaError_t launch_expand_batch(const BatchSeg* segs, const unsigned long long* chunk_begin, int nseg,
                                 unsigned long long total_chunks, const unsigned long long* keys,
                                 const unsigned long long* adj_all, unsigned long long* table,
