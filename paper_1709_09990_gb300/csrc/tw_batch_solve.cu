@@ -6,7 +6,11 @@
 // (Section 3.1), the block's warps taking the chunks of 32 states in turn, with
 // only block barriers between levels - until the treewidth is certified (yes
 // at tw, and no at tw-1 or tw equal to the lower bound), walks back through
-// its levels for the ordering, and takes the next graph.  The per-graph k
+// its levels for the ordering, and takes the next graph.  A block's levels are
+// bound by latency (four warps, block barriers), and the launch lasts as long as
+// its longest sweep: a graph of more than one_launch_n vertices is given up once
+// a run holds `limit` sets (the host's choice, with both sides' times, is in
+// run_batch_persistent).  The per-graph k
 // sweep starts at the lower bound, or at a proposed bound (learned-k), and
 // moves up on no and down on yes.  A graph whose levels outgrow the block's
 // workspace is marked and left to the single-graph path; nothing else leaves

@@ -237,8 +237,8 @@ __device__ __forceinline__ void graph_bounds(K* rows, const unsigned long long* 
   }
 }
 
-// Graphs of up to 64 vertices work on 64-bit rows: half the instructions of a
-// step and half the shared-memory words.
+// A chain of warp argmins per graph: latency.  Graphs of up to 64 vertices work
+// on 64-bit rows, half the instructions and shared-memory words of a step.
 __global__ void __launch_bounds__(kWarpsPerBlock * 32)
     bounds_kernel(const unsigned long long* __restrict__ adj, const int32_t* __restrict__ ns,
                   const int64_t* __restrict__ offs, int num_graphs, int32_t* out, float* feats, int lower_only) {
@@ -258,7 +258,8 @@ __global__ void __launch_bounds__(kWarpsPerBlock * 32)
 }
 
 // The two lower bounds of one graph of n vertices, a warp each: both are chains
-// of warp argmins, and a solve waits for them.
+// of warp argmins, and a solve waits for them (one after the other they take
+// 106 us for 70 vertices, 54 for 44; 43 for 44 side by side).
 __global__ void __launch_bounds__(64) lower_bounds_kernel(const unsigned long long* __restrict__ adj, int n,
                                                           int32_t* out) {
   __shared__ K128 sRows[2][128];

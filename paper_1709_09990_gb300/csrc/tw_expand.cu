@@ -18,12 +18,12 @@
 //     sector per load.  Pairs that need no search come first in the queue.
 //  3. New sets wait in shared memory and are appended to L_{i+1} with one atomic
 //     add per 200 or so: all adds of a level go to one counter.
-// The kernel is bound by instruction issue (62% of the issue slots at the peak
-// level of the geometric n=40 graph) and L2 round trips; the expand time of that
-// graph's 79.4 M sets is 7.7 ms, against 11.1 ms with a search per state (all
-// components of G[S] first, then the candidates) and slot-by-slot
-// compare-and-swaps, of which 3.4 ms went to lanes waiting for the warp's
-// longest probe sequence and to the counter.
+// The kernel is bound by the ALU pipe (67% at the peak level of the geometric
+// n=40 graph, issue 59%) and L2 round trips; the expand time of that graph's
+// 79.4 M sets is 7.0 ms, against 11.1 ms with a search per state (all components
+// of G[S] first, then the candidates), slot-by-slot compare-and-swaps, where a
+// warp waits for its longest probe sequence, and an add to the level's counter
+// per 128 pairs.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -196,7 +196,8 @@ __global__ void fingerprint_kernel(const K* __restrict__ keys, unsigned long lon
   }
 }
 
-// The levels of a finished run in one launch: blockIdx.y + 1 is the level, whose
+// The levels of a finished run in one launch (HBM read; with a launch, a copy and
+// a wait per level a 20-level decide took 0.35 ms longer): blockIdx.y + 1 is the level, whose
 // count keys lie at off; out[2 y], out[2 y + 1] += sum and xor.
 template <class K>
 __global__ void fingerprint_levels_kernel(const K* __restrict__ keys, const unsigned long long* __restrict__ off,

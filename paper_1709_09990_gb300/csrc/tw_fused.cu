@@ -9,7 +9,8 @@
 // consecutive decide runs of the sweep (k, k+1, ...) run at the same time,
 // one per group, so the sweep takes about as many level steps as its longest
 // run instead of their sum; a run stops as soon as a smaller k has answered yes
-// (the runs above tw are the large ones: on G(44, 0.5) they took 16 of 21 ms).  Within a group every block runs the same loop:
+// (the runs above tw are the large ones).  Within a group every block runs the
+// same loop:
 // expand level i (the group's blocks take the chunks of 32 states in turn,
 // the kernel body of tw_expand_core.cuh) while emptying the table the
 // previous level used, then one barrier of the group.  Every block reads the
@@ -18,6 +19,14 @@
 // tables alternate per group; all levels of a run stay in the group's arena
 // for the walk.  The answer is that of the sequential sweep: the smallest k
 // that answers yes, with every smaller k answering no.
+//
+// The launch is a chain of level steps of 4 to 8 us (the barrier 1.8 us, the
+// chunk's L2 round trips the rest) while levels are small, and bound like the
+// expand kernel when they hold 10^5 sets.  Whole solves, with the search per
+// state, waits for every run and a walk that scanned the levels -> now:
+// G(20, 0.3) 341 -> 243 us, a partial 8-tree of 34 vertices 1.42 -> 0.59 ms,
+// G(44, 0.5) 21.3 -> 1.40 ms, G(70, 0.8) (128-bit sets, as a graph-driven loop
+// before) 3.04 -> 1.03 ms.
 //
 // A run gives up (status "bail") when a level would not fit the arena or the
 // table, or when a table fills; the host then continues the sweep with its
