@@ -34,7 +34,7 @@ __device__ __forceinline__ unsigned long long home_slot(unsigned long long h, un
 // (both empty for S = {}), by a bitset flood fill over the adjacency rows in
 // shared memory.
 template <class K>
-__device__ __forceinline__ void min_component(const K S, const AdjRow<K>* __restrict__ sAdj, K& comp, K& bnd) {
+__host__ __device__ __forceinline__ void min_component(const K S, const AdjRow<K>* __restrict__ sAdj, K& comp, K& bnd) {
   comp = kzero<K>();
   K q = kzero<K>();
   K front = klsb(S);
@@ -70,7 +70,7 @@ struct Candidates {
   K done, search;
 };
 template <class K, bool kCanonical>
-__device__ __forceinline__ Candidates<K> cheap_candidates(const K S, const K comp0, const K b0,
+__host__ __device__ __forceinline__ Candidates<K> cheap_candidates(const K S, const K comp0, const K b0,
                                                           const AdjRow<K>* __restrict__ sAdj, const K valid, const K allowed,
                                                           const int k) {
   K cand = valid & allowed & ~S;
@@ -107,7 +107,7 @@ __device__ __forceinline__ Candidates<K> cheap_candidates(const K S, const K com
 //
 // vb is v's bit, nv its row.
 template <class K>
-__device__ __forceinline__ bool extension_feasible(const K S, const K comp0, const K b0, const K vb, const K nv,
+__host__ __device__ __forceinline__ bool extension_feasible(const K S, const K comp0, const K b0, const K vb, const K nv,
                                                    const AdjRow<K>* __restrict__ sAdj, const int k) {
   const K out = ~(S | vb);
   K q = nv;
@@ -672,7 +672,7 @@ __device__ __forceinline__ void expand_level(const ExpandParams<K>& p, AdjRow<K>
                                              const unsigned group_block = 0, const unsigned group_blocks = 0,
                                              K* out_tail = nullptr, const unsigned long long out_split = 0) {
   if (!kGroup) {
-    for (int i = threadIdx.x; i < p.n; i += blockDim.x) set_row(sAdj[i], p.adj[i], i);
+    fill_rows<K>(sAdj, p.adj, p.n, threadIdx.x, blockDim.x);
     __syncthreads();
   }
   const int lane = threadIdx.x & 31;

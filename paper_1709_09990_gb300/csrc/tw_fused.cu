@@ -239,7 +239,7 @@ __global__ void __launch_bounds__(kFusedWarps<K> * 32, 16 / kFusedWarps<K>)
   __shared__ unsigned int sSeen;
   __shared__ K128 sTdAdj[128];
   __shared__ int sPos[128];
-  for (int i = threadIdx.x; i < a.n; i += blockDim.x) set_row(sAdj[i], a.adj[i], i);
+  fill_rows<K>(sAdj, a.adj, a.n, threadIdx.x, blockDim.x);
   for (int j = threadIdx.x; j <= a.n; j += blockDim.x) sSets[j] = core::binom_capped(a.n, j, core::kSetsCap);
   __syncthreads();
   unsigned int round = 0, w_round = 0;  // this block's barriers on its group's and the grid's counter

@@ -59,9 +59,23 @@ template <> __host__ __device__ __forceinline__ K128 kfirst_n<K128>(int n) {
 }
 
 // ---- queries ----------------------------------------------------------------
-__device__ __forceinline__ int kpopc(uint32_t a) { return __popc(a); }
-__device__ __forceinline__ int kpopc(unsigned long long a) { return __popcll(a); }
-__device__ __forceinline__ int kpopc(K128 a) { return __popcll(a.lo) + __popcll(a.hi); }
+// (What the search of a level uses also compiles for the host, where the tests
+// run it.)
+__host__ __device__ __forceinline__ int kpopc(uint32_t a) {
+#ifdef __CUDA_ARCH__
+  return __popc(a);
+#else
+  return __builtin_popcount(a);
+#endif
+}
+__host__ __device__ __forceinline__ int kpopc(unsigned long long a) {
+#ifdef __CUDA_ARCH__
+  return __popcll(a);
+#else
+  return __builtin_popcountll(a);
+#endif
+}
+__host__ __device__ __forceinline__ int kpopc(K128 a) { return kpopc(a.lo) + kpopc(a.hi); }
 
 __host__ __device__ __forceinline__ bool kempty(uint32_t a) { return a == 0u; }
 __host__ __device__ __forceinline__ bool kempty(unsigned long long a) { return a == 0ull; }
@@ -80,23 +94,35 @@ __device__ __forceinline__ K128 kdrop_lowest(K128 a) {
 }
 
 // Lowest set bit of a as a one-bit set (a must be non-empty for an index).
-__device__ __forceinline__ uint32_t klsb(uint32_t a) { return a & (0u - a); }
-__device__ __forceinline__ unsigned long long klsb(unsigned long long a) { return a & (0ull - a); }
-__device__ __forceinline__ K128 klsb(K128 a) {
+__host__ __device__ __forceinline__ uint32_t klsb(uint32_t a) { return a & (0u - a); }
+__host__ __device__ __forceinline__ unsigned long long klsb(unsigned long long a) { return a & (0ull - a); }
+__host__ __device__ __forceinline__ K128 klsb(K128 a) {
   return a.lo ? K128{a.lo & (0ull - a.lo), 0ull} : K128{0ull, a.hi & (0ull - a.hi)};
 }
 
 // The vertices below the lowest element of a (every vertex when a is empty).
-__device__ __forceinline__ uint32_t kbelow_lowest(uint32_t a) { return (a - 1u) & ~a; }
-__device__ __forceinline__ unsigned long long kbelow_lowest(unsigned long long a) { return (a - 1ull) & ~a; }
-__device__ __forceinline__ K128 kbelow_lowest(K128 a) {
+__host__ __device__ __forceinline__ uint32_t kbelow_lowest(uint32_t a) { return (a - 1u) & ~a; }
+__host__ __device__ __forceinline__ unsigned long long kbelow_lowest(unsigned long long a) { return (a - 1ull) & ~a; }
+__host__ __device__ __forceinline__ K128 kbelow_lowest(K128 a) {
   return a.lo ? K128{(a.lo - 1ull) & ~a.lo, 0ull} : K128{~0ull, (a.hi - 1ull) & ~a.hi};
 }
 
 // Index of the only set bit of a one-bit set.
-__device__ __forceinline__ int kindex(uint32_t b) { return 31 - __clz(b); }
-__device__ __forceinline__ int kindex(unsigned long long b) { return 63 - __clzll(b); }
-__device__ __forceinline__ int kindex(K128 b) { return b.lo ? 63 - __clzll(b.lo) : 127 - __clzll(b.hi); }
+__host__ __device__ __forceinline__ int kindex(uint32_t b) {
+#ifdef __CUDA_ARCH__
+  return 31 - __clz(b);
+#else
+  return 31 - __builtin_clz(b);
+#endif
+}
+__host__ __device__ __forceinline__ int kindex(unsigned long long b) {
+#ifdef __CUDA_ARCH__
+  return 63 - __clzll(b);
+#else
+  return 63 - __builtin_clzll(b);
+#endif
+}
+__host__ __device__ __forceinline__ int kindex(K128 b) { return b.lo ? kindex(b.lo) : 64 + kindex(b.hi); }
 
 __device__ __forceinline__ bool ktest(uint32_t a, int v) { return (a >> v) & 1u; }
 __device__ __forceinline__ bool ktest(unsigned long long a, int v) { return (a >> v) & 1ull; }
@@ -113,12 +139,16 @@ __device__ __forceinline__ K128 kshfl(K128 a, int src) {
 
 // ---- rows in shared memory -----------------------------------------------------
 // Index of the highest set bit (a must be non-empty).
-__device__ __forceinline__ int khighest(uint32_t a) {
+__host__ __device__ __forceinline__ int khighest(uint32_t a) {
+#ifdef __CUDA_ARCH__
   int r;
   asm("bfind.u32 %0, %1;" : "=r"(r) : "r"(a));
   return r;
+#else
+  return 31 - __builtin_clz(a);
+#endif
 }
-__device__ __forceinline__ int khighest(unsigned long long a) {
+__host__ __device__ __forceinline__ int khighest(unsigned long long a) {
   const uint32_t hi = (uint32_t)(a >> 32);
   return khighest(hi ? hi : (uint32_t)a) + (hi ? 32 : 0);
 }
@@ -133,20 +163,31 @@ __device__ __forceinline__ int khighest(unsigned long long a) {
 // from pick(); own_bit() the bit of vertex v, whose row is a.
 template <class K> struct __align__(2 * sizeof(K)) AdjRow { K row, bit; };
 template <> struct AdjRow<K128> { K128 row; };
-template <class K> __device__ __forceinline__ int pick(const K set, K&) { return khighest(set); }
-template <> __device__ __forceinline__ int pick<K128>(const K128 set, K128& bit) {
+template <class K> __host__ __device__ __forceinline__ int pick(const K set, K&) { return khighest(set); }
+template <> __host__ __device__ __forceinline__ int pick<K128>(const K128 set, K128& bit) {
   bit = klsb(set);
   return kindex(bit);
 }
-template <class K> __device__ __forceinline__ K bit_of(const AdjRow<K>& a, const K) { return a.bit; }
-template <> __device__ __forceinline__ K128 bit_of<K128>(const AdjRow<K128>&, const K128 bit) { return bit; }
-template <class K> __device__ __forceinline__ K own_bit(const AdjRow<K>& a, const int) { return a.bit; }
-template <> __device__ __forceinline__ K128 own_bit<K128>(const AdjRow<K128>&, const int v) { return kbit<K128>(v); }
-__device__ __forceinline__ void set_row(AdjRow<uint32_t>& a, uint32_t row, int v) { a = {row, 1u << v}; }
-__device__ __forceinline__ void set_row(AdjRow<unsigned long long>& a, unsigned long long row, int v) {
+template <class K> __host__ __device__ __forceinline__ K bit_of(const AdjRow<K>& a, const K) { return a.bit; }
+template <> __host__ __device__ __forceinline__ K128 bit_of<K128>(const AdjRow<K128>&, const K128 bit) { return bit; }
+template <class K> __host__ __device__ __forceinline__ K own_bit(const AdjRow<K>& a, const int) { return a.bit; }
+template <> __host__ __device__ __forceinline__ K128 own_bit<K128>(const AdjRow<K128>&, const int v) { return kbit<K128>(v); }
+__host__ __device__ __forceinline__ void set_row(AdjRow<uint32_t>& a, uint32_t row, int v) { a = {row, 1u << v}; }
+__host__ __device__ __forceinline__ void set_row(AdjRow<unsigned long long>& a, unsigned long long row, int v) {
   a = {row, 1ull << v};
 }
-__device__ __forceinline__ void set_row(AdjRow<K128>& a, K128 row, int) { a.row = row; }
+__host__ __device__ __forceinline__ void set_row(AdjRow<K128>& a, K128 row, int) { a.row = row; }
+
+// Fills the rows of a search from the n rows at adj, this thread every step-th
+// from first on.  Every row that a bit of a set can name is written, those of
+// n and above as vertices without edges: the search loops take a visited vertex
+// out of their set with the bit that stands beside its row, so a row that holds
+// no bit would keep a set with a bit at or above n (tw_expand_level_static takes
+// its sets unchecked) in the loop for ever.
+template <class K>
+__host__ __device__ __forceinline__ void fill_rows(AdjRow<K>* rows, const K* adj, int n, int first, int step) {
+  for (int v = first; v < KeyTraits<K>::kBits; v += step) set_row(rows[v], v < n ? adj[v] : kzero<K>(), v);
+}
 
 // ---- hashing ----------------------------------------------------------------
 // 64-bit finaliser of MurmurHash3 (Appleby); the paper also hashes states with

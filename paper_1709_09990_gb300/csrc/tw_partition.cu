@@ -92,7 +92,7 @@ __global__ void __launch_bounds__(kWarps * 32, 6)
   __shared__ int sHist[kMaxRanges];
   __shared__ int sCursor[kMaxRanges];
   __shared__ unsigned long long sBase[kMaxRanges];
-  for (int i = threadIdx.x; i < p.n; i += blockDim.x) set_row(sAdj[i], p.adj[i], i);
+  fill_rows<K>(sAdj, p.adj, p.n, threadIdx.x, blockDim.x);
   __syncthreads();
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
