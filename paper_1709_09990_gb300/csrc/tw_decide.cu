@@ -225,6 +225,7 @@ int run_decide_ooc(tw_ctx* c, KeyClass kc, int n, int k, DecideResult* R, int st
   release(c, &c->pred);
   release(c, &c->cand_key);
   release(c, &c->cand_v);
+  release_fused(c);
   DevBuf* dev[2] = {&c->keys, &c->ooc_keys};
   const int load_pct = c->cfg.table_load_pct > 0 ? std::min(90, c->cfg.table_load_pct) : 75;
   const int max_probes = c->cfg.max_probes > 0 ? c->cfg.max_probes : 256;

@@ -97,7 +97,18 @@ int put_solution(tw_ctx* c, int n, int words, int32_t* order, int32_t* td_parent
 }
 
 size_t total_bytes(const tw_ctx* c) {
-  return c->keys.bytes + c->pred.bytes + c->table.bytes + c->cand_key.bytes + c->cand_v.bytes + c->ooc_keys.bytes;
+  return c->keys.bytes + c->pred.bytes + c->table.bytes + c->cand_key.bytes + c->cand_v.bytes + c->ooc_keys.bytes +
+         c->fused.bytes;
+}
+
+bool release_fused(tw_ctx* c) {
+  if (!c->fused.ptr) return false;
+  cudaStreamSynchronize(c->stream);
+  cudaFree(c->fused.ptr);
+  c->fused.ptr = nullptr;
+  c->fused.bytes = 0;
+  c->fused_clean = false;
+  return true;
 }
 
 // Takes bytes (rounded up to 256) of pinned, device-mapped host memory from
@@ -137,9 +148,12 @@ int host_take(tw_ctx* c, size_t bytes, char** out) {
 }
 
 // Grows b to at least need bytes, keeping its first keep bytes.  Growth is
-// geometric while the cap allows it.
+// geometric while the cap allows it.  The fused solve's buffer gives way to a
+// level loop that needs its room (the run that used it has ended by then).
 int grow(tw_ctx* c, DevBuf* b, size_t need, size_t keep) {
   if (need <= b->bytes) return TW_OK;
+  const bool may_release = b != &c->fused;
+  if (total_bytes(c) - b->bytes + need > c->mem_cap && may_release) release_fused(c);
   const size_t others = total_bytes(c) - b->bytes;
   if (others + need > c->mem_cap) return TW_ERR_CAPACITY;
   size_t want = std::max(need, b->bytes * 2);
@@ -148,7 +162,7 @@ int grow(tw_ctx* c, DevBuf* b, size_t need, size_t keep) {
   void* p = nullptr;
   if (cudaMalloc(&p, want) != cudaSuccess) {
     cudaGetLastError();
-    if (want == need) return TW_ERR_CAPACITY;
+    if (may_release) release_fused(c);
     want = (need + 255) & ~size_t(255);
     if (cudaMalloc(&p, want) != cudaSuccess) {
       cudaGetLastError();

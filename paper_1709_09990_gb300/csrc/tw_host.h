@@ -185,7 +185,11 @@ int put_from_device(tw_ctx* c, void* dst, const void* src_dev, size_t bytes);
 // mirror h_out (allocated on first use).
 int fetch_solution(tw_ctx* c);
 int put_solution(tw_ctx* c, int n, int words, int32_t* order, int32_t* td_parent, uint64_t* td_bags);
+// Device bytes of the context's grow-only buffers, which mem_cap bounds.
 size_t total_bytes(const tw_ctx* c);
+// Frees the buffer of the fused solve (false when there is none): it is scratch
+// of a finished launch, and a run that outgrew it needs the room under the cap.
+bool release_fused(tw_ctx* c);
 int grow(tw_ctx* c, DevBuf* b, size_t need, size_t keep);
 int host_take(tw_ctx* c, size_t bytes, char** out);
 int validate_rows(const uint64_t* rows, int n);
