@@ -107,7 +107,7 @@ bool release_fused(tw_ctx* c) {
   cudaFree(c->fused.ptr);
   c->fused.ptr = nullptr;
   c->fused.bytes = 0;
-  c->fused_clean = false;
+  c->fused_clean = 0;
   return true;
 }
 
