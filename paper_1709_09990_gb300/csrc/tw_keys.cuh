@@ -164,9 +164,15 @@ __host__ __device__ __forceinline__ int khighest(unsigned long long a) {
 template <class K> struct __align__(2 * sizeof(K)) AdjRow { K row, bit; };
 template <> struct AdjRow<K128> { K128 row; };
 template <class K> __host__ __device__ __forceinline__ int pick(const K set, K&) { return khighest(set); }
+// (For 128-bit sets by selects, the lowest vertex of the word that has one: with
+// a branch each for klsb and kindex a solve of G(70, 0.8) takes 1.00 ms instead
+// of 0.91, one of G(128, 0.96) 0.59 instead of 0.53.)
 template <> __host__ __device__ __forceinline__ int pick<K128>(const K128 set, K128& bit) {
-  bit = klsb(set);
-  return kindex(bit);
+  const bool low = set.lo != 0ull;
+  const unsigned long long w = low ? set.lo : set.hi;
+  const unsigned long long b = w & (0ull - w);
+  bit = K128{low ? b : 0ull, low ? 0ull : b};
+  return khighest(b) + (low ? 0 : 64);
 }
 template <class K> __host__ __device__ __forceinline__ K bit_of(const AdjRow<K>& a, const K) { return a.bit; }
 template <> __host__ __device__ __forceinline__ K128 bit_of<K128>(const AdjRow<K128>&, const K128 bit) { return bit; }
