@@ -269,7 +269,8 @@ int tw_solve(tw_ctx* ctx, const uint64_t* adj, int n, int* tw, int32_t* order,
  *                num_graphs proposed starting bounds: decide runs at
  *                round(k_hint) and round(k_hint)-1 and walks up or down from
  *                there until the answer is certified (yes at tw, no at tw-1).
- *   st         : out (or NULL): totals over all graphs.
+ *   st         : out (or NULL): totals over all graphs; a decide run that one
+ *                kernel gave up and the next one made again counts once.
  * Returns the worst per-graph status. */
 int tw_solve_batch(tw_ctx* ctx, const uint64_t* adj_concat, const int32_t* n,
                    const int64_t* row_offset, int num_graphs, int* tw, int32_t* orders,

@@ -34,6 +34,27 @@ void add_copy(std::vector<CopySeg>* list, unsigned long long src, unsigned long 
     list->push_back({src + at, dst + at, std::min(kCopyPiece, count - at)});
 }
 
+// What tw_stats reports of decide runs.
+struct RunCounts {
+  unsigned long long states = 0, candidates = 0, generated = 0, runs = 0;
+  void add(const RunCounts& r) {
+    states += r.states;
+    candidates += r.candidates;
+    generated += r.generated;
+    runs += r.runs;
+  }
+  // to st (or nowhere), and back to nothing
+  void move_to(tw_stats* st) {
+    if (st) {
+      st->states_expanded += states;
+      st->candidates += candidates;
+      st->generated += generated;
+      st->decide_runs += runs;
+    }
+    *this = RunCounts();
+  }
+};
+
 struct BGraph {
   int in_idx = 0;
   int n = 0;
@@ -48,6 +69,10 @@ struct BGraph {
   unsigned long long ocap_retry = 0;
   int tw = -1;
   int64_t order_off = 0;
+  // A run counts when it has ended: a graph that leaves the batch makes its
+  // present run again elsewhere, and its yes runs (held until the graph is done),
+  // but none of its no runs.
+  RunCounts run, held;
 };
 
 // Decide-only mode of run_batch (tw_decide_batch): every graph runs one
@@ -274,7 +299,8 @@ int run_batch(tw_ctx* c, const std::vector<HostGraph>& graphs, const std::vector
       copies.push_back({~0ull, B.atop, 1});
       x.levels.push_back({B.atop, 1});
       B.atop += 1;
-      if (st) st->decide_runs += 1;
+      x.run = RunCounts();
+      x.run.runs = 1;
     }
     if (!copies.empty()) {
       TW_CK(cudaMemcpyAsync(B.copies, copies.data(), copies.size() * sizeof(CopySeg), cudaMemcpyHostToDevice,
@@ -327,6 +353,7 @@ int run_batch(tw_ctx* c, const std::vector<HostGraph>& graphs, const std::vector
             if (dm->fp_xor) (*dm->fp_xor)[gi].push_back(fp[2 * q + 1]);
             ++q;
           }
+          x.run.move_to(st);
           x.tw = x.k;
           x.state = 1;
           x.levels.clear();
@@ -339,7 +366,8 @@ int run_batch(tw_ctx* c, const std::vector<HostGraph>& graphs, const std::vector
         if (x.state != 0) continue;
         const int last = (int)x.levels.size() - 1;
         if (x.levels.back().count == 0) {
-          record_answer(x, false);
+          x.run.move_to(st);
+          if (record_answer(x, false)) x.held.move_to(st);
           x.levels.clear();
           answered = true;
         } else if (last == x.n - x.k - 1) {
@@ -357,8 +385,10 @@ int run_batch(tw_ctx* c, const std::vector<HostGraph>& graphs, const std::vector
       // this stream)
       TW_LAUNCH(c, launch_walk_batch(B.walks, (int)walks.size(), B.lvl, B.akeys, B.apar, B.orders, c->stream));
       for (int j : walked) {
-        record_answer(B.g[j], true);
-        B.g[j].levels.clear();
+        BGraph& x = B.g[j];
+        x.held.add(x.run);
+        if (record_answer(x, true)) x.held.move_to(st);
+        x.levels.clear();
       }
       answered = true;
     }
@@ -470,11 +500,9 @@ int run_batch(tw_ctx* c, const std::vector<HostGraph>& graphs, const std::vector
       if (table_full || h.out_count > segs[s2].o_cap) continue;
       x.ocap_retry = 0;
       const int i = (int)x.levels.size() - 1;
-      if (st) {
-        st->states_expanded += segs[s2].in_count;
-        st->candidates += segs[s2].in_count * (unsigned long long)(x.n - i);
-        st->generated += h.generated;
-      }
+      x.run.states += segs[s2].in_count;
+      x.run.candidates += segs[s2].in_count * (unsigned long long)(x.n - i);
+      x.run.generated += h.generated;
       add_copy(&copies, segs[s2].o_off, B.atop, h.out_count);
       x.levels.push_back({B.atop, h.out_count});
       B.atop += h.out_count;

@@ -13,8 +13,8 @@
 // run_batch_persistent).  The per-graph k
 // sweep starts at the lower bound, or at a proposed bound (learned-k), and
 // moves up on no and down on yes.  A graph whose levels outgrow the block's
-// workspace is marked and left to the single-graph path; nothing else leaves
-// the device until the batch is done.
+// workspace is marked and left to the level-synchronous kernel (tw_batch.cu);
+// nothing else leaves the device until the batch is done.
 //
 // In decide mode every graph runs one decide at its own k and reports its
 // answer, level sizes and level fingerprints (tw_decide_batch).
@@ -33,6 +33,21 @@ using core::ExpandParams;
 using K = unsigned long long;
 constexpr unsigned kFull = 0xffffffffu;
 
+
+// What tw_stats reports of decide runs; thread 0 keeps them.  A run counts when it
+// has ended: the next kernel makes a run that outgrew the workspace again from
+// its empty set, and the yes runs of a graph that is left to it too, while the no
+// runs are not made again.
+struct RunCounts {
+  unsigned long long states, candidates, generated, runs;
+  __device__ void clear() { states = candidates = generated = runs = 0ull; }
+  __device__ void add(const RunCounts& r) {
+    states += r.states;
+    candidates += r.candidates;
+    generated += r.generated;
+    runs += r.runs;
+  }
+};
 
 // The block's view of its workspace.
 struct Work {
@@ -79,12 +94,17 @@ __device__ void block_fingerprint(const K* keys, unsigned long long count, unsig
 
 // decide(k) of one graph by one block into its workspace.  Returns false when
 // the levels outgrow the workspace; else *yes and *last (the final level).
-// With fp_sum / fp_xor (decide mode) the level fingerprints are written.
+// With fp_sum / fp_xor (decide mode) the level fingerprints are written.  *run gets
+// the run's counts.
 template <int kWarps>
 __device__ __noinline__ bool block_decide(const BatchSolveArgs& a, const K* adj, int n, int k, Work& w, AdjRow<K>* sAdj,
                              core::WarpScratch<K>* sScratch, const unsigned long long* sSets,
                              unsigned long long* sRed, bool* yes, int* last,
-                             unsigned long long* stats, unsigned long long* fp_sum, unsigned long long* fp_xor) {
+                             RunCounts* run, unsigned long long* fp_sum, unsigned long long* fp_xor) {
+  if (threadIdx.x == 0) {
+    run->clear();
+    run->runs = 1ull;
+  }
   for (int t = 0; t < 2; ++t) {
     for (unsigned long long j = threadIdx.x; j < w.dirty[t]; j += blockDim.x) w.table[t][j] = kones<K>();
     w.dirty[t] = 0;
@@ -155,10 +175,10 @@ __device__ __noinline__ bool block_decide(const BatchSolveArgs& a, const K* adj,
       w.dirty[t] = 0;
       __syncthreads();
     }
-    stats[0] += cnt;
-    stats[1] += cnt * (unsigned long long)(n - i);
-    stats[2] += gen;
     if (threadIdx.x == 0) {
+      run->states += cnt;
+      run->candidates += cnt * (unsigned long long)(n - i);
+      run->generated += gen;
       w.off[i + 1] = out_off;
       w.cnt[i + 1] = got;
     }
@@ -197,8 +217,8 @@ __global__ void __launch_bounds__(kWarps * 32, 24 / kWarps) batch_solve_kernel(c
   w.ctr = a.ctr + slot;
   w.off = a.level_off + slot * 130;
   w.cnt = a.level_cnt + slot * 130;
-  unsigned long long stats[3] = {0ull, 0ull, 0ull};
-  unsigned long long runs = 0;
+  __shared__ RunCounts sRun, sYes, sTotal;  // the run, the graph's yes runs, the block's counted runs
+  if (threadIdx.x == 0) sTotal.clear();
   for (;;) {
     if (threadIdx.x == 0) sGraph = (int)atomicAdd(a.next_graph, 1u);
     __syncthreads();
@@ -214,9 +234,9 @@ __global__ void __launch_bounds__(kWarps * 32, 24 / kWarps) batch_solve_kernel(c
       unsigned long long* fs = a.fp_sum ? a.fp_sum + (size_t)g * 129 : nullptr;
       unsigned long long* fx = a.fp_xor ? a.fp_xor + (size_t)g * 129 : nullptr;
       const bool ok = block_decide<kWarps>(a, adj, n, a.k_start[g], w, sAdj, sScratch, sSets, sRed, &yes, &last,
-                                           stats, fs, fx);
-      ++runs;
+                                           &sRun, fs, fx);
       if (threadIdx.x == 0) {
+        if (ok) sTotal.add(sRun);
         a.status[g] = ok ? 0 : 2;
         a.yes[g] = yes ? 1 : 0;
         a.last[g] = last;
@@ -231,10 +251,11 @@ __global__ void __launch_bounds__(kWarps * 32, 24 / kWarps) batch_solve_kernel(c
     int k = a.k_start[g];
     int yes_min = INT_MAX, no_max = lb - 1, yes_in_arena = -1;
     bool ok = true;
+    if (threadIdx.x == 0) sYes.clear();
     for (;;) {
-      ok = block_decide<kWarps>(a, adj, n, k, w, sAdj, sScratch, sSets, sRed, &yes, &last, stats, nullptr, nullptr);
-      ++runs;
+      ok = block_decide<kWarps>(a, adj, n, k, w, sAdj, sScratch, sSets, sRed, &yes, &last, &sRun, nullptr, nullptr);
       if (!ok) break;
+      if (threadIdx.x == 0) (yes ? sYes : sTotal).add(sRun);
       if (yes) {
         yes_min = min(yes_min, k);
         yes_in_arena = k;
@@ -247,9 +268,9 @@ __global__ void __launch_bounds__(kWarps * 32, 24 / kWarps) batch_solve_kernel(c
     }
     if (ok && yes_in_arena != yes_min) {
       // the last run was a no: run the yes at tw again for its levels
-      ok = block_decide<kWarps>(a, adj, n, yes_min, w, sAdj, sScratch, sSets, sRed, &yes, &last, stats, nullptr,
+      ok = block_decide<kWarps>(a, adj, n, yes_min, w, sAdj, sScratch, sSets, sRed, &yes, &last, &sRun, nullptr,
                                 nullptr);
-      ++runs;
+      if (threadIdx.x == 0) sYes.add(sRun);
     }
     if (!ok) {
       if (threadIdx.x == 0) {
@@ -261,16 +282,17 @@ __global__ void __launch_bounds__(kWarps * 32, 24 / kWarps) batch_solve_kernel(c
     }
     if (a.orders) core::walk_block<K>(w.arena, w.pred, w.off, w.cnt, last, n, a.orders + a.order_off[g], &sWalk, &sFound);
     if (threadIdx.x == 0) {
+      sTotal.add(sYes);
       a.status[g] = 0;
       a.tw[g] = yes_min;
     }
     __syncthreads();
   }
   if (threadIdx.x == 0) {
-    atomicAdd(&a.totals[0], stats[0]);
-    atomicAdd(&a.totals[1], stats[1]);
-    atomicAdd(&a.totals[2], stats[2]);
-    atomicAdd(&a.totals[3], runs);
+    atomicAdd(&a.totals[0], sTotal.states);
+    atomicAdd(&a.totals[1], sTotal.candidates);
+    atomicAdd(&a.totals[2], sTotal.generated);
+    atomicAdd(&a.totals[3], sTotal.runs);
   }
 }
 
