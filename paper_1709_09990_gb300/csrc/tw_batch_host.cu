@@ -20,6 +20,13 @@ namespace host {
 // expand_batch_kernel.  A graph whose level would exceed kEvictStates leaves
 // the batch and is solved afterwards by the single-graph path, which sizes
 // its buffers for large levels.
+//
+// Every level of a running graph stays in the batch's arena until its run ends.
+// The arena, the table and the output lists keep within what the memory cap
+// leaves: a step takes as many graphs as its table and lists have room for, and
+// when the arena cannot grow half of the running graphs wait and start their
+// present run again later.  A graph that runs alone is given what the device
+// has; only when the device refuses it too does it go to the single-graph path.
 constexpr double kEvictStates = double(1 << 21);
 constexpr unsigned long long kStepSlots = 1ull << 27;   // table slots per step
 constexpr unsigned long long kStepOut = 1ull << 26;     // output states per step
@@ -63,7 +70,7 @@ struct BGraph {
   int k = -1;
   int yes_min = 1 << 30;
   int no_max = -1;
-  int state = 0;  // 0 running, 1 done, 2 evicted
+  int state = 0;  // 0 running, 1 done, 2 evicted, 3 waiting for memory
   std::vector<LevelRec> levels;
   double table_mult = 1.0;
   unsigned long long ocap_retry = 0;
@@ -116,16 +123,64 @@ struct BatchRun {
   WalkSeg* walks = nullptr;
   unsigned long long* lvl = nullptr;
   int32_t* orders = nullptr;
-  size_t nslots_meta = 0;
-  std::vector<void*> owned;
+  size_t budget = 0;      // device bytes that arena, table and output lists may hold
+  int admitted = 0;       // graphs that may run at once
 
-  explicit BatchRun(tw_ctx* cc) : c(cc) {}
+  explicit BatchRun(tw_ctx* cc) : c(cc) { set_budget(); }
   ~BatchRun() {
     cudaStreamSynchronize(c->stream);
     for (void* p : {(void*)adj, (void*)akeys, (void*)apar, (void*)table, (void*)okeys, (void*)opar, (void*)segs,
                     (void*)cbeg, (void*)ctr, (void*)copies, (void*)walks, (void*)lvl, (void*)orders})
       if (p) cudaFree(p);
     cudaGetLastError();
+  }
+
+  void set_budget() { budget = c->mem_cap > total_bytes(c) ? c->mem_cap - total_bytes(c) : 0; }
+  int running() const {
+    int r = 0;
+    for (const BGraph& x : g) r += x.state == 0 ? 1 : 0;
+    return r;
+  }
+  // May the buffers hold this many more bytes?  A graph alone is not held to the
+  // budget for what it cannot do without.
+  bool fits(size_t more, bool needed) const {
+    return acap * 12 + tcap * 8 + ocap * 12 + more <= budget || (needed && running() <= 1);
+  }
+
+  // After a refused allocation: gives the batch room or fewer graphs to run.  The
+  // buffers of the single-graph path go first (they are scratch between calls),
+  // then half of the running graphs wait; a graph that the device refuses even
+  // alone leaves the batch.
+  void make_way() {
+    const size_t held = total_bytes(c);
+    release_scratch(c);
+    if (total_bytes(c) < held) {
+      set_budget();
+      return;
+    }
+    const int now = running();
+    admitted = std::max(1, now / 2);
+    int kept = 0;
+    for (BGraph& x : g) {
+      if (x.state != 0 || (now > 1 && kept++ < admitted)) continue;
+      x.state = now > 1 ? 3 : 2;
+      if (!x.levels.empty()) {  // (a run under way starts again at its own k)
+        x.k0 = x.k;
+        x.k = -1;
+      }
+      x.levels.clear();
+      x.run = RunCounts();
+      x.ocap_retry = 0;
+    }
+  }
+  // Lets waiting graphs run while fewer than admitted do.
+  void admit() {
+    int now = running();
+    for (BGraph& x : g)
+      if (x.state == 3 && now < admitted) {
+        x.state = 0;
+        ++now;
+      }
   }
 
   size_t live_states() const {
@@ -137,36 +192,55 @@ struct BatchRun {
   }
 
   // Makes room for need more arena states, compacting the live levels of
-  // running graphs into a fresh arena when the current one is full.
+  // running graphs into a fresh arena when the current one is full: one of twice
+  // what is needed, or of just that.  TW_ERR_CAPACITY when there is no room for
+  // either.
   int arena_room(unsigned long long need) {
     if (atop + need <= acap) return TW_OK;
     const unsigned long long live = live_states();
-    const unsigned long long want = std::max<unsigned long long>({acap, 2 * (live + need), 1ull << 20});
     unsigned long long* nk = nullptr;
     uint32_t* np = nullptr;
-    int rc = dev_alloc(&nk, want);
-    if (rc == TW_OK) rc = dev_alloc(&np, want);
-    if (rc != TW_OK) {
+    unsigned long long want = 0;
+    int rc = TW_ERR_CAPACITY;
+    for (const unsigned long long w : {std::max<unsigned long long>({acap, 2 * (live + need), 1ull << 20}), live + need}) {
+      want = w;
+      if (!fits(w * 12, w == live + need)) continue;
+      rc = dev_alloc(&nk, w);
+      if (rc == TW_OK) rc = dev_alloc(&np, w);
+      if (rc == TW_OK) break;
       if (nk) cudaFree(nk);
-      return rc;
+      nk = nullptr;
     }
+    if (rc != TW_OK) return rc;
     std::vector<CopySeg> cs;
     unsigned long long top = 0;
-    for (BGraph& x : g) {
+    for (const BGraph& x : g) {
       if (x.state != 0) continue;
-      for (LevelRec& l : x.levels) {
+      for (const LevelRec& l : x.levels) {
         add_copy(&cs, l.off, top, l.count);
-        l.off = top;
         top += l.count;
       }
     }
-    if (!cs.empty()) {
-      CopySeg* d = nullptr;
-      if ((rc = dev_alloc(&d, cs.size()))) return rc;
+    CopySeg* d = nullptr;
+    if (!cs.empty() && (rc = dev_alloc(&d, cs.size()))) {
+      cudaFree(nk);
+      cudaFree(np);
+      return rc;
+    }
+    if (d) {
       TW_CK(cudaMemcpyAsync(d, cs.data(), cs.size() * sizeof(CopySeg), cudaMemcpyHostToDevice, c->stream));
       TW_LAUNCH(c, launch_copy_segments(d, (int)cs.size(), akeys, apar, nk, np, c->stream));
       TW_CK(cudaStreamSynchronize(c->stream));
       cudaFree(d);
+    }
+    // (the levels move only now that nothing can be refused any more)
+    top = 0;
+    for (BGraph& x : g) {
+      if (x.state != 0) continue;
+      for (LevelRec& l : x.levels) {
+        l.off = top;
+        top += l.count;
+      }
     }
     TW_CK(cudaStreamSynchronize(c->stream));
     if (akeys) cudaFree(akeys);
@@ -178,17 +252,37 @@ struct BatchRun {
     return TW_OK;
   }
 
-  template <class T>
-  int ensure(T** p, unsigned long long* cap, unsigned long long need) {
-    if (need <= *cap && *p) return TW_OK;
+  // Table and output lists of the step (their contents need not be kept);
+  // TW_ERR_CAPACITY when there is no room for them.
+  int table_room(unsigned long long need) {
+    if (need <= tcap) return TW_OK;
     TW_CK(cudaStreamSynchronize(c->stream));
-    if (*p) cudaFree(*p);
-    *p = nullptr;
-    const unsigned long long want = std::max<unsigned long long>(need, *cap * 2);
-    int rc = dev_alloc(p, want);
-    if (rc) return rc;
-    *cap = want;
-    return TW_OK;
+    const unsigned long long twice = 2 * tcap;
+    if (table) cudaFree(table);
+    table = nullptr;
+    tcap = 0;
+    for (const unsigned long long want : {std::max(need, twice), need}) {
+      if (!fits(want * 8, want == need) || dev_alloc(&table, want) != TW_OK) continue;
+      tcap = want;
+      return TW_OK;
+    }
+    return TW_ERR_CAPACITY;
+  }
+  int list_room(unsigned long long need) {
+    if (need <= ocap) return TW_OK;
+    TW_CK(cudaStreamSynchronize(c->stream));
+    const unsigned long long twice = 2 * ocap;
+    for (const unsigned long long want : {std::max(need, twice), need}) {
+      if (okeys) cudaFree(okeys);
+      if (opar) cudaFree(opar);
+      okeys = nullptr;
+      opar = nullptr;
+      ocap = 0;
+      if (!fits(want * 12, want == need) || dev_alloc(&okeys, want) != TW_OK || dev_alloc(&opar, want) != TW_OK) continue;
+      ocap = want;
+      return TW_OK;
+    }
+    return TW_ERR_CAPACITY;
   }
 };
 
@@ -283,15 +377,22 @@ int run_batch(tw_ctx* c, const std::vector<HostGraph>& graphs, const std::vector
   std::vector<unsigned long long> lvl;
   std::vector<int> seg_graph;
   size_t rr = 0;
+  B.admitted = G;
 
   for (int step = 0;; ++step) {
+    B.admit();
     // 1. start a run (level 0 = {empty set}) for graphs without one
     copies.clear();
     {
       unsigned long long starting = 0;
       for (const BGraph& x : B.g)
         if (x.state == 0 && x.levels.empty()) ++starting;
-      if (starting && (rc = B.arena_room(starting))) return rc;  // before any offset is handed out
+      rc = starting ? B.arena_room(starting) : TW_OK;  // before any offset is handed out
+      if (rc == TW_ERR_CAPACITY) {
+        B.make_way();
+        continue;
+      }
+      if (rc) return rc;
     }
     for (BGraph& x : B.g) {
       if (x.state != 0 || !x.levels.empty()) continue;
@@ -399,6 +500,10 @@ int run_batch(tw_ctx* c, const std::vector<HostGraph>& graphs, const std::vector
     seg_graph.clear();
     unsigned long long tsum = 0, osum = 0, chunks = 0;
     int running = 0;
+    // (a quarter of the budget each for the table and the lists, the rest for the
+    // arena and its successor)
+    const unsigned long long max_slots = std::min<unsigned long long>(kStepSlots, B.budget / 32);
+    const unsigned long long max_out = std::min<unsigned long long>(kStepOut, B.budget / 48);
     for (int t = 0; t < G; ++t) {
       const int j = (int)((rr + t) % G);
       BGraph& x = B.g[j];
@@ -431,7 +536,7 @@ int run_batch(tw_ctx* c, const std::vector<HostGraph>& graphs, const std::vector
                        : std::min<unsigned long long>(
                              (unsigned long long)std::ceil(std::min(bound, std::max(table_est * 3.0, 1024.0))),
                              slots / 10ull * 9ull + 64ull);
-      if (!segs.empty() && (tsum + slots > kStepSlots || osum + oc > kStepOut)) continue;
+      if (!segs.empty() && (tsum + slots > max_slots || osum + oc > max_out)) continue;
       BatchSeg sg;
       sg.in_off = cur.off;
       sg.in_count = cur.count;
@@ -451,17 +556,21 @@ int run_batch(tw_ctx* c, const std::vector<HostGraph>& graphs, const std::vector
       osum += oc;
     }
     rr = (rr + 1) % (size_t)G;
-    if (running == 0) break;
+    if (running == 0) {
+      bool waiting = false;
+      for (const BGraph& x : B.g) waiting = waiting || x.state == 3;
+      if (waiting) continue;
+      break;
+    }
     if (segs.empty()) continue;  // evictions only
     cbeg.push_back(chunks);
-    if ((rc = B.ensure(&B.table, &B.tcap, tsum + 2))) return rc;
-    {
-      unsigned long long cap_o = B.ocap;
-      if ((rc = B.ensure(&B.okeys, &cap_o, osum))) return rc;
-      unsigned long long cap_p = B.ocap;
-      if ((rc = B.ensure(&B.opar, &cap_p, osum))) return rc;
-      B.ocap = std::min(cap_o, cap_p);
+    rc = B.table_room(tsum + 2);
+    if (rc == TW_OK) rc = B.list_room(osum);
+    if (rc == TW_ERR_CAPACITY) {
+      B.make_way();
+      continue;
     }
+    if (rc) return rc;
     const int nseg = (int)segs.size();
     TW_CK(cudaMemcpyAsync(B.segs, segs.data(), nseg * sizeof(BatchSeg), cudaMemcpyHostToDevice, c->stream));
     TW_CK(cudaMemcpyAsync(B.cbeg, cbeg.data(), (nseg + 1) * 8, cudaMemcpyHostToDevice, c->stream));
@@ -491,7 +600,12 @@ int run_batch(tw_ctx* c, const std::vector<HostGraph>& graphs, const std::vector
       }
       need += h.out_count;
     }
-    if ((rc = B.arena_room(need))) return rc;
+    rc = B.arena_room(need);
+    if (rc == TW_ERR_CAPACITY) {  // (the graphs that go on build these levels again)
+      B.make_way();
+      continue;
+    }
+    if (rc) return rc;
     copies.clear();
     for (int s2 = 0; s2 < nseg; ++s2) {
       BGraph& x = B.g[seg_graph[s2]];

@@ -183,14 +183,6 @@ int ooc_host_buffer(tw_ctx* c, int hb, size_t bytes, char** dptr) {
   return TW_OK;
 }
 
-void release(tw_ctx* c, DevBuf* b) {
-  if (!b->ptr) return;
-  cudaStreamSynchronize(c->stream);
-  cudaFree(b->ptr);
-  b->ptr = nullptr;
-  b->bytes = 0;
-}
-
 // Allocates b with exactly bytes (rounded up to 256); false when the cap or
 // the device refuses.
 bool alloc_exact(tw_ctx* c, DevBuf* b, size_t bytes) {

@@ -101,14 +101,24 @@ size_t total_bytes(const tw_ctx* c) {
          c->fused.bytes;
 }
 
+void release(tw_ctx* c, DevBuf* b) {
+  if (!b->ptr) return;
+  cudaStreamSynchronize(c->stream);
+  cudaFree(b->ptr);
+  b->ptr = nullptr;
+  b->bytes = 0;
+}
+
 bool release_fused(tw_ctx* c) {
   if (!c->fused.ptr) return false;
-  cudaStreamSynchronize(c->stream);
-  cudaFree(c->fused.ptr);
-  c->fused.ptr = nullptr;
-  c->fused.bytes = 0;
+  release(c, &c->fused);
   c->fused_clean = 0;
   return true;
+}
+
+void release_scratch(tw_ctx* c) {
+  release_fused(c);
+  for (DevBuf* b : {&c->keys, &c->pred, &c->table, &c->cand_key, &c->cand_v, &c->ooc_keys}) release(c, b);
 }
 
 // Takes bytes (rounded up to 256) of pinned, device-mapped host memory from

@@ -189,6 +189,9 @@ size_t total_bytes(const tw_ctx* c);
 // Frees the buffer of the fused solve (false when there is none): it is scratch
 // of a finished launch, and a run that outgrew it needs the room under the cap.
 bool release_fused(tw_ctx* c);
+void release(tw_ctx* c, DevBuf* b);
+// Frees every buffer that total_bytes counts.  They hold nothing between calls.
+void release_scratch(tw_ctx* c);
 int grow(tw_ctx* c, DevBuf* b, size_t need, size_t keep);
 int host_take(tw_ctx* c, size_t bytes, char** out);
 int validate_rows(const uint64_t* rows, int n);
