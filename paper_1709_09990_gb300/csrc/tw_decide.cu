@@ -1069,26 +1069,30 @@ int run_fused(tw_ctx* c, const HostGraph& g, KeyClass kc, int k0, int k_last, De
   constexpr int kGroups = 3;
   static_assert(kGroups <= kFusedMaxGroups, "the fused launch holds at most kFusedMaxGroups groups");
   const int G = std::max(1, std::min(kGroups, k_last - k0 + 1));
-  // (128-bit states: half the states, the same bytes)
-  constexpr unsigned long long kStates128 = 1ull << 19;
-  const unsigned long long A =
-      c->cfg.fused_states > 0 ? (unsigned long long)c->cfg.fused_states : (kc == kKey128 ? kStates128 : 2 * kStates128);
-  const unsigned long long T = 2 * A + 1024;
+  // By default 128-bit states get half the states and table slots of the others,
+  // so that every buffer of both widths has the same place and size: a context
+  // that solves graphs of up to 64 and of more vertices in turn finds its tables
+  // empty (emptying them at each change took 26 us of a 200 us solve).  (Where the
+  // tables lie matters by itself: 8 KB further apart, a 20-vertex solve takes 201
+  // instead of 193 us.)
+  const bool given = c->cfg.fused_states > 0, wide = kc == kKey128;
+  const unsigned long long A = given ? (unsigned long long)c->cfg.fused_states : 1ull << (wide ? 19 : 20);
+  const unsigned long long T = 2 * A + (wide && !given ? 512 : 1024);
   const size_t st_bytes = (sizeof(FusedState) + 255) & ~size_t(255);
-  const size_t unit = kc == kKey128 ? 16 : 8;  // bytes per slot and key (32-bit states: room for 64)
-  // (the same bytes per table for both widths by default, see below)
-  const size_t tb = ((c->cfg.fused_states > 0 ? (size_t)T * unit : (2 * kStates128 + 1024) * 16) + 255) & ~size_t(255);
+  const size_t unit = wide ? 16 : 8;  // bytes per slot and key (32-bit states: room for 64)
+  const size_t tb = ((size_t)T * unit + 255) & ~size_t(255);
   const size_t kb = ((size_t)A * unit + 255) & ~size_t(255);
-  const size_t pb = ((size_t)A * 4 + 255) & ~size_t(255);
-  // the groups' states side by side, then every group's tables, then their keys
-  // and parents: the tables of both widths lie at the same place, so a context
-  // that solves graphs of up to 64 and of more vertices in turn finds them empty
-  // (with the tables between the keys it emptied 100 MB at each change)
-  const size_t tables_bytes = (size_t)kGroups * 2 * tb;
-  const size_t need = (size_t)kGroups * (st_bytes + kb + pb) + tables_bytes;
+  const size_t pb = ((size_t)(given ? A : 1ull << 20) * 4 + 255) & ~size_t(255);
+  // the groups' states side by side, then each group's tables, keys and parents
+  const size_t group_bytes = 2 * tb + kb + pb;
+  const size_t need = (size_t)kGroups * (st_bytes + group_bytes);
   *status = 0;
+  if (c->fused_layout != group_bytes) {
+    c->fused_clean = false;  // the groups' tables lie elsewhere
+    c->fused_layout = group_bytes;
+  }
   if (c->fused.bytes < need) {
-    c->fused_clean = 0;
+    c->fused_clean = false;
     int rc = grow(c, &c->fused, need, 0);
     if (rc == TW_ERR_CAPACITY) return TW_OK;  // no room under the cap: the level loop runs instead
     if (rc) return rc;
@@ -1102,7 +1106,6 @@ int run_fused(tw_ctx* c, const HostGraph& g, KeyClass kc, int k0, int k_last, De
     }
   }
   char* base = static_cast<char*>(c->fused.ptr);
-  char* tables = base + kGroups * st_bytes;
   SmallLayout L;
   FusedLaunch f;
   f.kc = kc;
@@ -1118,25 +1121,24 @@ int run_fused(tw_ctx* c, const HostGraph& g, KeyClass kc, int k0, int k_last, De
   f.lb_dev = lb_dev;
   for (int j = 0; j < kFusedMaxGroups; ++j) {
     const size_t at = (size_t)std::min(j, kGroups - 1);
-    char* lists = tables + tables_bytes + at * (kb + pb);
+    char* gbase = base + kGroups * st_bytes + at * group_bytes;
     f.st[j] = reinterpret_cast<FusedState*>(base + at * st_bytes);
-    f.table0[j] = tables + 2 * at * tb;
-    f.table1[j] = tables + (2 * at + 1) * tb;
-    f.keys[j] = lists;
-    f.parent_of[j] = reinterpret_cast<uint32_t*>(lists + kb);
+    f.table0[j] = gbase;
+    f.table1[j] = gbase + tb;
+    f.keys[j] = gbase + 2 * tb;
+    f.parent_of[j] = reinterpret_cast<uint32_t*>(gbase + 2 * tb + kb);
   }
   f.arena_cap = A;
   f.table_cap = T;
   f.order = reinterpret_cast<int32_t*>(small_at(c, L.order));
   f.parent = reinterpret_cast<int32_t*>(small_at(c, L.parent));
   f.bags = reinterpret_cast<unsigned long long*>(small_at(c, L.bags));
-  if (c->fused_clean < tables_bytes) {
-    // a new buffer, one a launch left early, or larger tables than the last
-    // launch's: empty the rest of the tables (all ones) once; launches that run to
-    // their end leave them empty
-    TW_CK(cudaMemsetAsync(tables + c->fused_clean, 0xff, tables_bytes - c->fused_clean, c->stream));
+  if (!c->fused_clean) {
+    // a new buffer, or one a launch left early: empty every group's tables
+    // (all ones) once; launches that run to their end leave them empty
+    for (int j = 0; j < kGroups; ++j) TW_CK(cudaMemsetAsync(f.table0[j], 0xff, 2 * tb, c->stream));
+    c->fused_clean = true;
   }
-  c->fused_clean = 0;
   f.tables_clean = 1;
   TW_CK(cudaMemsetAsync(base, 0, G * st_bytes, c->stream));
   const bool timed = c->cfg.time_kernels != 0;
@@ -1151,9 +1153,7 @@ int run_fused(tw_ctx* c, const HostGraph& g, KeyClass kc, int k0, int k_last, De
   TW_CK(cudaStreamSynchronize(c->stream));
   const FusedState& h = *c->h_fused;
   c->h_out_fresh = want_out && h.error == 0u && h.status == 1 && h.tw >= 0;
-  // a launch that ran to its end empties the tables it used (its keys lie after
-  // them)
-  c->fused_clean = h.error == 0u ? tables_bytes : 0;
+  c->fused_clean = h.error == 0u;  // a launch that ran to its end empties the tables it used
   if (h.error) return TW_ERR_TIMEOUT;  // a barrier wait gave up
   *status = h.status;
   k0 = h.k_start;  // (raised by the device lower bounds when given)

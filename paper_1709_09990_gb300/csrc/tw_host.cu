@@ -112,7 +112,7 @@ void release(tw_ctx* c, DevBuf* b) {
 bool release_fused(tw_ctx* c) {
   if (!c->fused.ptr) return false;
   release(c, &c->fused);
-  c->fused_clean = 0;
+  c->fused_clean = false;
   return true;
 }
 

@@ -99,7 +99,8 @@ struct tw_ctx {
   // fused small solves: state, two tables and the level arena in one buffer,
   // a pinned mirror of the state, and the graphs whose fused run gave up
   DevBuf fused;
-  size_t fused_clean = 0;    // bytes of its tables, from the first one on, that hold empty slots only
+  size_t fused_layout = 0;   // bytes of a group in it (another layout: other places)
+  bool fused_clean = false;  // every table slot of the fused buffer is empty
   FusedState* h_fused = nullptr;
   bool h_out_fresh = false;        // h_out holds the solution of the solve under way
   unsigned char* h_up = nullptr;   // pinned staging of upload_graph
