@@ -81,3 +81,21 @@ def test_graphs_that_exceed_the_cap_together(batch_kernel, cap_mb):
     used = (mem.first - mem.least) // MB
     assert used <= max(cap_mb, 288) + 32, used
     assert res["stats"]["expand_launches"] > ref["stats"]["expand_launches"]
+
+
+@pytest.mark.parametrize("cap_mb", [0, 8])
+def test_small_graphs_in_the_persistent_kernel(cap_mb):
+    # one graph of 16 vertices among larger ones (its runs may hold 2^16 sets, the
+    # others' 2^12), and a batch of them under a cap that leaves a block 2^12:
+    # graphs that outgrow that go on in the level-synchronous kernel
+    mixed = [gg.gnp(16, 0.3, 1)] + [gg.mixed_graph(9100 + j, 17, 28, j % 2 == 0) for j in range(30)]
+    small = [gg.gnp(16, 0.15 + 0.01 * j, 60 + j) for j in range(40)]
+    with context(mem_cap_bytes=cap_mb * MB) as c:
+        for graphs in (mixed, small):
+            exp = [oracle.solve(a, want_order=False)["tw"] for a in graphs]
+            res = c.solve_batch(graphs)
+            assert res["status"] == 0 and res["tw"].tolist() == exp
+            pos = 0
+            for adj, t in zip(graphs, exp):
+                assert oracle.width_elim(adj, res["orders"][pos: pos + len(adj)].tolist()) == t
+                pos += len(adj)

@@ -29,3 +29,12 @@ def test_widths_in_turn_find_empty_tables(states):
                 for st in (one["stats"], three["stats"]):
                     for key in ("level_size", "fp_sum", "fp_xor"):
                         assert st[key] == exp[key], (key, turn, len(adj))
+
+
+@pytest.mark.parametrize("adj", [gg.path(128), gg.path(70), gg.gnp(70, 0.8, 110), gg.workload_gnp20()],
+                         ids=["path128", "path70", "gnp70", "gnp20"])
+def test_launches_do_not_grow_with_the_levels(adj):
+    # the bounds, the fused launch and one launch for all level fingerprints
+    with context(fingerprints=True) as c:
+        for _ in range(2):
+            assert c.solve(adj, want_td=True)["stats"]["kernel_launches"] <= 3
