@@ -1091,6 +1091,7 @@ int run_fused(tw_ctx* c, const HostGraph& g, KeyClass kc, int k0, int k_last, De
     c->fused_clean = false;  // the groups' tables lie elsewhere
     c->fused_layout = group_bytes;
   }
+  if (c->count_fused && total_bytes(c) > c->mem_cap) release_fused(c);
   if (c->fused.bytes < need) {
     c->fused_clean = false;
     int rc = grow(c, &c->fused, need, 0);

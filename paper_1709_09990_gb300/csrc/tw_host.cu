@@ -98,7 +98,7 @@ int put_solution(tw_ctx* c, int n, int words, int32_t* order, int32_t* td_parent
 
 size_t total_bytes(const tw_ctx* c) {
   return c->keys.bytes + c->pred.bytes + c->table.bytes + c->cand_key.bytes + c->cand_v.bytes + c->ooc_keys.bytes +
-         c->fused.bytes;
+         (c->count_fused ? c->fused.bytes : 0);
 }
 
 void release(tw_ctx* c, DevBuf* b) {
@@ -159,12 +159,14 @@ int host_take(tw_ctx* c, size_t bytes, char** out) {
 
 // Grows b to at least need bytes, keeping its first keep bytes.  Growth is
 // geometric while the cap allows it.  The fused solve's buffer gives way to a
-// level loop that needs its room (the run that used it has ended by then).
+// level loop that needs its room (the run that used it has ended by then): under
+// the cap where it counts, and where the device has no more memory.
 int grow(tw_ctx* c, DevBuf* b, size_t need, size_t keep) {
   if (need <= b->bytes) return TW_OK;
   const bool may_release = b != &c->fused;
-  if (total_bytes(c) - b->bytes + need > c->mem_cap && may_release) release_fused(c);
-  const size_t others = total_bytes(c) - b->bytes;
+  auto held_without = [&]() { return total_bytes(c) - (b == &c->fused && !c->count_fused ? 0 : b->bytes); };
+  if (c->count_fused && may_release && held_without() + need > c->mem_cap) release_fused(c);
+  const size_t others = held_without();
   if (others + need > c->mem_cap) return TW_ERR_CAPACITY;
   size_t want = std::max(need, b->bytes * 2);
   if (others + want > c->mem_cap) want = need;
@@ -242,6 +244,7 @@ char* small_at(tw_ctx* c, size_t off) { return static_cast<char*>(c->small.ptr) 
 // copy of both from pinned memory.
 int upload_graph(tw_ctx* c, const HostGraph& g, KeyClass kc) {
   SmallLayout L;
+  c->count_fused = kc == kKey128;
   if (!c->h_up) {
     if (cudaHostAlloc(reinterpret_cast<void**>(&c->h_up), L.walk, cudaHostAllocDefault) != cudaSuccess) {
       c->h_up = nullptr;

@@ -101,6 +101,7 @@ struct tw_ctx {
   DevBuf fused;
   size_t fused_layout = 0;   // bytes of a group in it (another layout: other places)
   bool fused_clean = false;  // every table slot of the fused buffer is empty
+  bool count_fused = false;  // total_bytes counts it (the call's graph has more than 64 vertices)
   FusedState* h_fused = nullptr;
   bool h_out_fresh = false;        // h_out holds the solution of the solve under way
   unsigned char* h_up = nullptr;   // pinned staging of upload_graph
@@ -185,10 +186,14 @@ int put_from_device(tw_ctx* c, void* dst, const void* src_dev, size_t bytes);
 // mirror h_out (allocated on first use).
 int fetch_solution(tw_ctx* c);
 int put_solution(tw_ctx* c, int n, int words, int32_t* order, int32_t* td_parent, uint64_t* td_bags);
-// Device bytes of the context's grow-only buffers, which mem_cap bounds.
+// Device bytes of the context's grow-only buffers, which mem_cap bounds.  The fused
+// solve's buffer is among them in calls on graphs of more than 64 vertices; for
+// others a context holds it besides (with it counted there too, a small cap sent
+// small graphs to the level loop once a large one had filled it: 288 graphs of the
+// batch workload one by one under 0.5 GB took 0.42 s instead of 0.15).
 size_t total_bytes(const tw_ctx* c);
 // Frees the buffer of the fused solve (false when there is none): it is scratch
-// of a finished launch, and a run that outgrew it needs the room under the cap.
+// of a finished launch.
 bool release_fused(tw_ctx* c);
 void release(tw_ctx* c, DevBuf* b);
 // Frees every buffer that total_bytes counts.  They hold nothing between calls.
