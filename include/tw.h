@@ -57,7 +57,12 @@ typedef struct tw_ctx tw_ctx;
 typedef struct {
   int device;             /* CUDA device ordinal                                  */
   int fingerprints;       /* 1: fill level_fp_sum / level_fp_xor in tw_stats     */
-  size_t mem_cap_bytes;   /* device bytes libtw may hold; 0 = 150 GB or 90% free  */
+  size_t mem_cap_bytes;   /* device bytes the levels and tables of a call may hold;
+                             0 = 150 GB or 90% of the free memory.  Besides it: the
+                             fused solve's buffer for n <= 64 (138 MB, freed when
+                             the device has no more), a persistent batch's arenas
+                             above a quarter of it (168 KB a block), and the levels
+                             of a tw_solve_batch's level-synchronous steps.       */
   void* stream;           /* cudaStream_t to run on; NULL = a stream of libtw's  */
   int block_threads;      /* expand kernel block size; 0 = autotuned/default     */
   int table_load_pct;     /* hash table target load in percent; 0 = default (50) */
@@ -95,7 +100,8 @@ typedef struct {
                              one into their slice of the table, which is emptied
                              in L2 just before and dropped from L2 without a
                              write-back after, so the table stays out of DRAM.
-                             0 = 256 MB (the default), -1 = never, -2 = every
+                             0 = 256 MB (the default), -1 = never (faster on the
+                             levels measured, see tw_decide.cu), -2 = every
                              level.  Results are unchanged.                     */
   int mmw_prune;          /* 1 = Section 3.3: a state whose remaining graph has a
                              minor-min-width bound (second-smallest degree of each
@@ -140,11 +146,12 @@ typedef struct {
                              disjoint_paths, mmw_prune or spill_levels.  Results
                              are unchanged.                                      */
   int batch_kernel;       /* tw_solve_batch / tw_decide_batch: 0 = one persistent
-                             launch for the whole batch, each block solving one
-                             graph at a time from a device queue (the default);
-                             1 = level-synchronous steps, one launch per step for
-                             the current level of every running graph.  Results
-                             are unchanged.                                      */
+                             launch, each block solving one graph at a time from
+                             a device queue, then level-synchronous steps for the
+                             graphs that outgrew a block's arena (the default);
+                             1 = level-synchronous steps alone, one launch per
+                             step for the current level of every running graph.
+                             Results are unchanged.                              */
   int host_cap_mb;        /* out_of_core: pinned host memory, in MB, that levels
                              may occupy; 0 = 85% of the host's physical memory  */
   int batch_arena_states; /* persistent batched kernel: states each block's arena
@@ -251,8 +258,8 @@ int tw_solve(tw_ctx* ctx, const uint64_t* adj, int n, int* tw, int32_t* order,
 
 /* Many graphs of uneven size in one batched run (the Section 3.1 sweep for
  * each graph).  By default one persistent launch
- * solves the graphs from a device queue, a block per graph (the whole k sweep,
- * certification and walk on the device); graphs whose decide runs outgrow a
+ * solves the small graphs from a device queue, a block per graph (the whole k
+ * sweep, certification and walk on the device); graphs whose decide runs outgrow a
  * block's arena (batch_arena_states) continue in level-synchronous steps that
  * expand the current level of every such graph over the whole GPU, and graphs
  * that outgrow those, or have n > 64, are solved one at a time
@@ -340,7 +347,8 @@ int tw_mlp_train(tw_ctx* ctx, float* params, const float* x, const float* y, int
  * Its hash table and counters live in a fixed static device array of 16 MiB
  * + 256 bytes inside libtw, held by every GPU that loads the library until
  * the process exits.
- *   d_in_keys  : device, n_in 64-bit keys of level i (bit v = vertex v).
+ *   d_in_keys  : device, n_in 64-bit keys of level i (bit v = vertex v; not
+ *                checked, a bit at or above n is a vertex without edges).
  *                The output is level i+1 when the input is the whole of
  *                level i: like tw_decide, each set is extended only by the
  *                vertices of the component of S u {v} that holds its lowest

@@ -28,7 +28,11 @@ namespace host {
 
 // Table size above which a level takes the partitioned insert: by default
 // tables of more than 256 MB (about twice the L2), where the direct kernel's
-// compare-and-swaps go to DRAM.
+// accesses go to DRAM.  The line was drawn when the direct kernel probed slot by
+// slot with compare-and-swaps (level 8 of the partial 10-tree 5.9 ms against 4.4).
+// Since it probes whole sectors it is the faster one on that graph (whole calls up
+// to level 8, 9 and 10: 4.4, 16.0 and 51 ms with partition_table_mb = -1, 5.5, 21.6
+// and 76 ms by default), so -1 is the better setting for such levels.
 unsigned long long partition_threshold_bytes(const tw_ctx* c) {
   if (c->cfg.partition_table_mb == -2) return 0ull;
   if (c->cfg.partition_table_mb < 0) return ~0ull;

@@ -18,8 +18,8 @@
 //     sector per load.  Pairs that need no search come first in the queue.
 //  3. New sets wait in shared memory and are appended to L_{i+1} with one atomic
 //     add per 200 or so: all adds of a level go to one counter.
-// The kernel is bound by the ALU pipe (67% at the peak level of the geometric
-// n=40 graph, issue 59%) and L2 round trips; the expand time of that graph's
+// The kernel is bound by the ALU pipe (65% at the peak level of the geometric
+// n=40 graph, issue 60%) and L2 round trips; the expand time of that graph's
 // 79.4 M sets is 7.0 ms, against 11.1 ms with a search per state (all components
 // of G[S] first, then the candidates), slot-by-slot compare-and-swaps, where a
 // warp waits for its longest probe sequence, and an add to the level's counter

@@ -424,9 +424,9 @@ __device__ __forceinline__ void flush_stage(WarpScratch<K>& w, int& staged, cons
   __syncwarp();
 }
 
-// Slot of the sector in which key stands or may be put: the first of its slots
-// from `from` on that may be empty, kPresent when key comes before that, kFull
-// when every slot holds another key.
+// Slot of the sector in which key may be put: the first of its slots from `from`
+// on that may be empty, kSlotPresent when key comes before that, kSlotNone when
+// every slot holds another key.
 constexpr int kSlotPresent = -1, kSlotNone = -2;
 template <class K>
 __device__ __forceinline__ int find_slot(const Sector<K>& s, const K key, const int from) {

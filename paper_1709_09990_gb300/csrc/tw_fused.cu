@@ -26,7 +26,7 @@
 // state, waits for every run and a walk that scanned the levels -> now:
 // G(20, 0.3) 341 -> 243 us, a partial 8-tree of 34 vertices 1.42 -> 0.59 ms,
 // G(44, 0.5) 21.3 -> 1.40 ms, G(70, 0.8) (128-bit sets, as a graph-driven loop
-// before) 3.04 -> 1.03 ms.
+// before) 3.04 -> 0.92 ms.
 //
 // A run gives up (status "bail") when a level would not fit the arena or the
 // table, or when a table fills; the host then continues the sweep with its

@@ -96,7 +96,7 @@ struct tw_ctx {
   // out-of-core decide runs: two pinned, device-mapped host buffers that hold
   // the levels that do not fit the device (reused from run to run)
   HostChunk ooc_host[2] = {{nullptr, nullptr, 0}, {nullptr, nullptr, 0}};
-  // fused small solves: state, two tables and the level arena in one buffer,
+  // fused small solves: three groups' states, tables and level arenas in one buffer,
   // a pinned mirror of the state, and the graphs whose fused run gave up
   DevBuf fused;
   size_t fused_layout = 0;   // bytes of a group in it (another layout: other places)
@@ -179,12 +179,12 @@ bool is_device_ptr(const void* p);
 int fetch(void* dst_host, const void* src, size_t bytes);
 int put(tw_ctx* c, void* dst, const void* src_host, size_t bytes);
 int put_from_device(tw_ctx* c, void* dst, const void* src_dev, size_t bytes);
-// The ordering, tree-decomposition parents and bags of a solve from the small
-// buffer into the caller's pointers (each host, device or NULL) with one
-// stream synchronisation.
 // Enqueues the copy of the small buffer's order .. bags region into the pinned
 // mirror h_out (allocated on first use).
 int fetch_solution(tw_ctx* c);
+// The ordering, tree-decomposition parents and bags of a solve from the small
+// buffer into the caller's pointers (each host, device or NULL) with one
+// stream synchronisation.
 int put_solution(tw_ctx* c, int n, int words, int32_t* order, int32_t* td_parent, uint64_t* td_bags);
 // Device bytes of the context's grow-only buffers, which mem_cap bounds.  The fused
 // solve's buffer is among them in calls on graphs of more than 64 vertices; for

@@ -33,8 +33,8 @@ struct ExpandLaunch {
   const void* adj;               // n rows, one key each
   int n;
   int k;
-  void* table;                   // power-of-two slots, all set to the empty key
-  unsigned long long table_slots;
+  void* table;                   // table_slots slots, all set to the empty key, 32-byte aligned (it
+  unsigned long long table_slots;  // is probed in 32-byte sectors; at least one, a rest is not used)
   int max_probes;
   void* out_keys;                // L_{i+1} keys (capacity out_cap)
   uint8_t* out_pred;             // predecessor vertex of each L_{i+1} state

@@ -266,9 +266,15 @@ __device__ __forceinline__ K128 kcas(K128* p, K128 cmp, K128 val) {
   return old;
 }
 
-// One 32-byte sector of a hash table, read with one access that goes to the L2
-// (other SMs write the table during a level).  Words are read whole; the two
-// halves of a 128-bit key may be of different times.
+// One 32-byte sector of a hash table (32-byte aligned), read with one access that
+// goes to the L2 (other SMs write the table during a level).  Words are read whole;
+// the two halves of a 128-bit key may be of different times.  Such a torn key, one
+// half of the set being written and one half still all ones, never equals a set
+// that is looked for, because all sets of one table have the same number of
+// vertices: equal to it, a set would have 64 of them in the half that reads as all
+// ones, and as many as the set being written only if that one has all 64 there too
+// and is the same set.  A table that held sets of several levels could not be probed
+// this way.
 template <class K> struct Sector { static constexpr int kSlots = 32 / (int)sizeof(K); K x[kSlots]; };
 __device__ __forceinline__ void kload_sector(const uint32_t* p, Sector<uint32_t>& s) {
   asm volatile("ld.relaxed.gpu.global.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"

@@ -1,4 +1,5 @@
-// Partitioned insert for levels whose hash table is far larger than L2.
+// Partitioned insert for levels whose hash table is far larger than L2 (above 256
+// MB by default; see partition_threshold_bytes for both sides' times).
 //
 // A compare-and-swap into a table that lives in DRAM costs a random 32-byte
 // sector read and, for a winner, a write-back; on GB300 such random accesses
