@@ -27,7 +27,9 @@ namespace host {
 // given what the device has; only when the device refuses it too does it go to the
 // single-graph path.  In decide mode the buffers keep within what the memory cap
 // leaves, and a step takes as many graphs as its table and lists have room for
-// (those graphs ran one at a time under the cap before they came here); a solve's
+// (those graphs ran one at a time under the cap before they came here: 288 graphs of
+// 16 to 48 vertices took 335 ms; under a cap of 512 MB they take 58 ms, under 64 MB
+// 277, with room for all at once 24); a solve's
 // are held to the device's memory only (the labels of 2000 training graphs under a
 // cap of 0.5 GB take 1.7 s; 4.7 s with these buffers and the fused solve's under it
 // too).
